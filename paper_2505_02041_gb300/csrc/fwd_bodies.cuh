@@ -175,17 +175,27 @@ template <class A, int C> struct TraceTile {
     }
 };
 
-// Trace of ray shape R from the probe whose tile offset is `base`; su / sv
-// are the tile strides along the frame's u and v axes.  Pieces J .. END-1
-// are unrolled at compile time.
-template <int P, int C, int J, int END>
-__device__ __forceinline__ void trace_pieces(const TraceTile<typename Prec<P>::A, C> &tt, int base, int su, int sv,
+// Tile steps along the axes of frame Q, known at compile time so that every
+// piece's shared-memory address is the probe's plus a constant, and the rays
+// of a column are picked by its residue mod 4 instead of ray by ray: the
+// kernel is bound by instruction issue (69 % of the slots at 1024^2), and this
+// cut it from 56.2 to 52.5 us there (C = 3, fp32) and from 189.5 to 177 us at
+// 2048^2.
+template <int Q> struct TraceFrame {
+    static constexpr int sgn = (Q == 0 || Q == 2) ? 1 : -1;   // image step along u
+    static constexpr int su = sgn * (Q < 2 ? 1 : TR_PITCH), sv = Q < 2 ? TR_PITCH : 1;
+};
+
+// Trace of ray shape R in frame Q from the probe whose tile offset is `base`.
+// Pieces J .. END-1 are unrolled at compile time.
+template <int P, int C, int Q, int J, int END>
+__device__ __forceinline__ void trace_pieces(const TraceTile<typename Prec<P>::A, C> &tt, int base,
                                              typename Prec<P>::A (&L)[C], typename Prec<P>::A &Tacc,
                                              typename Prec<P>::A &tau) {
     using A = typename Prec<P>::A;
     if constexpr (J < END) {
         using pc = PieceAt<J>;
-        const int o = base + pc::du * su + pc::dv * sv;
+        const int o = base + (pc::du * TraceFrame<Q>::su + pc::dv * TraceFrame<Q>::sv);
         const typename TraceTile<A, C>::V2 p = tt.tw[pc::cls * TR_PLANE + o];
         A t = p.x, w = p.y, em[C], sg;
         tt.emis(o, em, sg);
@@ -198,23 +208,79 @@ __device__ __forceinline__ void trace_pieces(const TraceTile<typename Prec<P>::A
         for (int c = 0; c < C; ++c) L[c] = fma(wt, em[c], L[c]);
         Tacc *= t;
         if constexpr (Prec<P>::LOG) tau = fma(sg, A(pc::full ? 2 : 1) * class_len<A>(pc::cls), tau);
-        trace_pieces<P, C, J + 1, END>(tt, base, su, sv, L, Tacc, tau);
+        trace_pieces<P, C, Q, J + 1, END>(tt, base, L, Tacc, tau);
     }
 }
 
-template <int P, int C, int R>
-__device__ __forceinline__ void trace_store(const Plan &pl, const TraceTile<typename Prec<P>::A, C> &tt, int q,
-                                            int nmax, int u, int v, int base, int su, int sv) {
+// The ray's entry, at the row of direction 0 of its column (entry v) plus k rows.
+template <int P, int C, int Q, int R>
+__device__ __forceinline__ void trace_store(const TraceTile<typename Prec<P>::A, C> &tt, char *col, long long G, int Vs,
+                                            int v, int base) {
     using A = typename Prec<P>::A;
-    using ray = RayAt<R>;
-    if (ray::n > nmax || (u & ((1 << ray::n) - 1)) || !t_live(ray::n, u >> ray::n, ray::k)) return;
-    Iv<P, C> iv;
+    using SL = typename Prec<P>::SL;
+    using ST = typename Prec<P>::ST;
+    A L[C];
 #pragma unroll
-    for (int c = 0; c < C; ++c) iv.L[c] = A(0);
+    for (int c = 0; c < C; ++c) L[c] = A(0);
     A Tacc = A(1), tau = A(0);
-    trace_pieces<P, C, ray::begin, ray::end>(tt, base, su, sv, iv.L, Tacc, tau);
-    iv.t = Prec<P>::LOG ? tau : Tacc;
-    TLevel<P, C>(pl, q, ray::n).store(u >> ray::n, ray::k, v, iv);
+    trace_pieces<P, C, Q, RayAt<R>::begin, RayAt<R>::end>(tt, base, L, Tacc, tau);
+    char *row = col + RayAt<R>::k * G;
+    SL *pl = reinterpret_cast<SL *>(row) + v;
+#pragma unroll
+    for (int c = 0; c < C; ++c) pl[c * Vs] = from_acc<SL>(L[c]);
+    reinterpret_cast<ST *>(row + (size_t)C * Vs * sizeof(SL))[v] = from_acc<ST>(Prec<P>::LOG ? tau : Tacc);
+}
+
+// The live rays (t_live) of the probe at frame column u >= 1: at odd u those
+// of T_0, at u = 2 mod 4 those of T_1, at u = 0 mod 4 the even directions of
+// T_1 and T_2.
+template <int P, int C, int Q>
+__device__ __forceinline__ void trace_column(const Plan &pl, const TraceTile<typename Prec<P>::A, C> &tt, int u, int v,
+                                             int base) {
+    const QuadGeom &g = pl.q[Q];
+    const int Vs = g.Vs;
+    const long long G = TLevel<P, C>(pl, Q, 0).G;
+    if (u & 1) {
+        char *c0 = pl.arena + g.Toff[0] + (long long)(2 * u) * G;
+        trace_store<P, C, Q, 0>(tt, c0, G, Vs, v, base);
+        trace_store<P, C, Q, 1>(tt, c0, G, Vs, v, base);
+        return;
+    }
+    if (g.N >= 1) {
+        char *c1 = pl.arena + g.Toff[1] + (long long)(3 * (u >> 1)) * G;
+        trace_store<P, C, Q, 2>(tt, c1, G, Vs, v, base);
+        if (u & 2) trace_store<P, C, Q, 3>(tt, c1, G, Vs, v, base);
+        trace_store<P, C, Q, 4>(tt, c1, G, Vs, v, base);
+    }
+    if (!(u & 2) && g.N >= 2) {
+        char *c2 = pl.arena + g.Toff[2] + (long long)(5 * (u >> 2)) * G;
+        trace_store<P, C, Q, 5>(tt, c2, G, Vs, v, base);
+        trace_store<P, C, Q, 6>(tt, c2, G, Vs, v, base);
+        trace_store<P, C, Q, 7>(tt, c2, G, Vs, v, base);
+        trace_store<P, C, Q, 8>(tt, c2, G, Vs, v, base);
+        trace_store<P, C, Q, 9>(tt, c2, G, Vs, v, base);
+    }
+}
+
+// Columns 8 i + ((warp + i) mod 8), i0 <= i < i1, of frame Q for the tile.
+template <int P, int C, int Q>
+__device__ __forceinline__ void trace_frame(const Plan &pl, const TraceTile<typename Prec<P>::A, C> &tt, int x0, int y0,
+                                            int i0, int i1) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    constexpr bool xu = Q < 2;                          // frame u runs along image x
+    const int tu = xu ? x0 : y0, tv = xu ? y0 : x0;     // tile origin along u / v axes
+    const int ext_u = xu ? pl.W : pl.H;
+    const int v = tv + lane;
+    if (v >= pl.q[Q].V) return;
+#pragma unroll 1
+    for (int i = i0; i < i1; ++i) {
+        const int c = 8 * i + ((warp + i) & 7);
+        if (tu + c >= ext_u) continue;
+        const int u = TraceFrame<Q>::sgn > 0 ? tu + c : ext_u - 1 - (tu + c);
+        if (u < 1) continue;                            // column 0 is dead
+        const int base = xu ? (TR_HALO + lane) * TR_PITCH + TR_HALO + c : (TR_HALO + c) * TR_PITCH + TR_HALO + lane;
+        trace_column<P, C, Q>(pl, tt, u, v, base);
+    }
 }
 
 // T_0..T_min(2,N) of the selected quadrant frames for one 32 x 32 image
@@ -222,18 +288,29 @@ __device__ __forceinline__ void trace_store(const Plan &pl, const TraceTile<type
 // frame's u axis (one column of every residue mod 4, so the warps get equal
 // shares of the level-1 and level-2 probes); its lanes run along v, so every
 // T store is a 128-byte coalesced row segment in every frame.
+// part / parts: on grids of few tiles a tile's work is cut into `parts` blocks
+// (16: one frame and one of its four column groups; 4: one frame; 2: a pair of
+// frames), each staging the tile.
 // With tme / tms (fp32 inputs), the region is fetched by TMA tensor copies;
 // a copy wait that gives up records its code in the plan's status word and
 // leaves the tile's T entries unwritten.
 template <int P, int C>
 __device__ __forceinline__ void body_trace012(const Plan &pl, const float *__restrict__ e, const float *__restrict__ s,
                                               const double *__restrict__ ed, const double *__restrict__ sd, int qmask,
-                                              int bx, int by, unsigned char *tr_smem,
+                                              int bx, int by, unsigned char *tr_smem, int part = 0, int parts = 1,
                                               const CUtensorMap *tme = nullptr, const CUtensorMap *tms = nullptr) {
     using A = typename Prec<P>::A;
     TraceTile<A, C> tt(tr_smem);
     const int W = pl.W, H = pl.H;
     const int x0 = bx * TR_TILE, y0 = by * TR_TILE;
+    int i0 = 0, i1 = TR_TILE / 8;
+    if (parts == 2) qmask &= 3 << (2 * part);
+    if (parts >= 4) qmask &= 1 << (part & 3);
+    if (parts == 16) {
+        i0 = part >> 2;
+        i1 = i0 + 1;
+    }
+    if (qmask == 0) return;
     if constexpr (P == P_FP64) {
         tt.stage(W, H, x0, y0, ed, sd);
     } else {
@@ -249,35 +326,10 @@ __device__ __forceinline__ void body_trace012(const Plan &pl, const float *__res
         }
     }
     __syncthreads();
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int q = 0; q < 4; ++q) {
-        if (!((qmask >> q) & 1)) continue;
-        const QuadGeom &g = pl.q[q];
-        const int nmax = g.N < 2 ? g.N : 2;
-        const bool xu = q < 2;                              // frame u runs along image x
-        const int tu = xu ? x0 : y0, tv = xu ? y0 : x0;     // tile origin along u / v axes
-        const int ext_u = xu ? W : H;
-        const int v = tv + lane;
-        const int sgn = (q == 0 || q == 2) ? 1 : -1;        // image step along u
-        const int su = sgn * (xu ? 1 : TR_PITCH), sv = xu ? TR_PITCH : 1;
-        for (int i = 0; i < TR_TILE / 8; ++i) {
-            const int c = 8 * i + ((warp + i) & 7);
-            if (tu + c >= ext_u || v >= g.V) continue;
-            const int u = (q == 0 || q == 2) ? tu + c : ext_u - 1 - (tu + c);
-            const int base = xu ? (TR_HALO + lane) * TR_PITCH + TR_HALO + c
-                                : (TR_HALO + c) * TR_PITCH + TR_HALO + lane;
-            trace_store<P, C, 0>(pl, tt, q, nmax, u, v, base, su, sv);
-            trace_store<P, C, 1>(pl, tt, q, nmax, u, v, base, su, sv);
-            trace_store<P, C, 2>(pl, tt, q, nmax, u, v, base, su, sv);
-            trace_store<P, C, 3>(pl, tt, q, nmax, u, v, base, su, sv);
-            trace_store<P, C, 4>(pl, tt, q, nmax, u, v, base, su, sv);
-            trace_store<P, C, 5>(pl, tt, q, nmax, u, v, base, su, sv);
-            trace_store<P, C, 6>(pl, tt, q, nmax, u, v, base, su, sv);
-            trace_store<P, C, 7>(pl, tt, q, nmax, u, v, base, su, sv);
-            trace_store<P, C, 8>(pl, tt, q, nmax, u, v, base, su, sv);
-            trace_store<P, C, 9>(pl, tt, q, nmax, u, v, base, su, sv);
-        }
-    }
+    if (qmask & 1) trace_frame<P, C, 0>(pl, tt, x0, y0, i0, i1);
+    if (qmask & 2) trace_frame<P, C, 1>(pl, tt, x0, y0, i0, i1);
+    if (qmask & 4) trace_frame<P, C, 2>(pl, tt, x0, y0, i0, i1);
+    if (qmask & 8) trace_frame<P, C, 3>(pl, tt, x0, y0, i0, i1);
 }
 
 // T_n(p, k) from T_{n-1}; p = (x 2^n, v).  Near operand at column 2x, far

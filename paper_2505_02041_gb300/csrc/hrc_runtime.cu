@@ -109,6 +109,7 @@ size_t build_plan(int W, int H, int C, int cascades, int prec, size_t off, Plan 
     pl.mthreads = 128;
     pl.vmajor = 0;
     pl.mdown = 0;
+    pl.solo = 1;
     pl.bulk_limit_ns = 2000000000LL;   // 2 s
     pl.bulk_extra_tx = 0;
     const size_t SLb = sl_bytes(prec), STb = st_bytes(prec);
@@ -1688,6 +1689,7 @@ hrc_status build_batched_plans(hrc_ctx *ctx, int prec) {
     for (int i = 0; i < ctx->nscenes; ++i) {
         off = build_plan(ctx->Ws[i], ctx->Hs[i], ctx->C, ctx->cascades, prec, off, ctx->bplans[i], true);
         ctx->bplans[i].arena = ctx->arena;
+        ctx->bplans[i].solo = ctx->nscenes == 1;
         ctx->bplans[i].sched = 0;
         ctx->bplans[i].mgroups = 1;
         ctx->bplans[i].mthreads = 128;

@@ -15,8 +15,8 @@ __global__ void __launch_bounds__(256) k_trace012(Plan pl, const float *__restri
                                                   int qmask, const __grid_constant__ CUtensorMap tme,
                                                   const __grid_constant__ CUtensorMap tms, int use_tma) {
     extern __shared__ __align__(128) unsigned char tr_smem[];
-    body_trace012<P, C>(pl, e, s, ed, sd, qmask, blockIdx.x, blockIdx.y, tr_smem, use_tma ? &tme : nullptr,
-                        use_tma ? &tms : nullptr);
+    body_trace012<P, C>(pl, e, s, ed, sd, qmask, blockIdx.x, blockIdx.y, tr_smem, blockIdx.z, gridDim.z,
+                        use_tma ? &tme : nullptr, use_tma ? &tms : nullptr);
 }
 
 // Row and v-block of this block: the launch grid is (rows, v-blocks), or
@@ -224,6 +224,16 @@ static cudaError_t fwd_impl(const Plan &pl, const RayTable &rt, const void *e, c
                 if ((qm >> q) & 1)
                     for (int n = 0; n <= 2; ++n) by += bytes_T(pl, q, n);
             dim3 grid((pl.W + TR_TILE - 1) / TR_TILE, (pl.H + TR_TILE - 1) / TR_TILE);
+            // Grids of few tiles: a tile's rays take one block about 12 us
+            // whatever the grid, so its work is cut into blocks until they
+            // cover the SMs (about two per SM); each part stages the tile
+            // again, so grids that fill the GPU take whole tiles.  fp32,
+            // parts 1 / 2 / 4 / 16 (trace alone, us): 64^2 13.0 / 10.4 / 9.2 /
+            // 8.6, 256^2 13.2 / 11.1 / 10.7 / 17.9, 384^2 C = 3 15.4 / 14.4 /
+            // 18.0 / 34.8, 512^2 C = 3 19.1 / 22.8 / 24.7 / 53.9.  Not in a
+            // batch, whose scenes share the GPU.
+            const unsigned tiles = grid.x * grid.y;
+            if (pl.solo) grid.z = tiles <= 19 ? 16 : (tiles <= 76 ? 4 : (tiles <= 152 ? 2 : 1));
             rec->begin(K_TRACE012, 0, by);
             CUtensorMap me, ms;
             std::memset(&me, 0, sizeof(me));

@@ -315,3 +315,14 @@ def test_maximum_extent_forward_and_backward(W, H):
     with pytest.raises(_lib.HRCError) as ex:
         HRC(W + 1 if W > H else W, H + 1 if H > W else H, 1)
     assert ex.value.status == _lib.HRC_EINVAL
+
+
+@pytest.mark.parametrize("W,H", [(601, 30), (640, 32), (608, 125), (2464, 32), (606, 256), (1630, 95), (3, 33)])
+def test_trace_parts_on_grids_of_few_tiles(W, H):
+    """The direct trace cuts a tile's rays into 16, 4, 2 or 1 blocks on grids
+    of up to 19, 76, 152 and more tiles: sizes on either side of each line
+    (with odd extents), fp32 against the oracle."""
+    require_gpu()
+    e, s = scenes.random_scene(W, H, 1, 95)
+    _, F = _gpu_F(e, s)
+    assert_fp32(F, oracle.fluence(e, s))
