@@ -389,10 +389,15 @@ __device__ __forceinline__ void body_adj_merge_up(const Plan &pl, const RowSplit
 // ---------------------------------------------------------------------------
 
 // Probe box of ray shape R for a tile of PT_U x PT_V frame pixels: the probes
-// (spacing S = 2^n along u) whose ray reaches the tile lie in
-// u in [u0 - S, u0 + PT_U) (PT_U / S + 1 aligned columns) and
+// whose ray reaches the tile lie in u in [u0 - 2^n, u0 + PT_U) and
 // v in [v0 - dvhi, v0 + PT_V - dvlo), dv of the shape in [dvlo, dvhi] (one
-// sign: a ray is monotone in v).
+// sign: a ray is monotone in v).  Only live probes (t_live) are in the box:
+// columns u = OF mod SP, PT_U / SP + 1 of them -- odd u for T_0, u = 2 mod 4
+// for the odd direction of T_1, else every 2^n-th.  (Taking every 2^n-th
+// column, dead ones with zero slots, cost 282 us at 1024^2 and 1036 at 2048^2,
+// C = 3, against 267 and 978.)
+constexpr int shape_spacing(int R) { return R < 2 ? 2 : (R == 3 || R >= 5 ? 4 : 2); }
+constexpr int shape_offset(int R) { return R < 2 ? 1 : (R == 3 ? 2 : 0); }
 constexpr int shape_dv_min(int R) {
     int m = 0;
     for (int j = kShapes.start[R]; j < kShapes.start[R + 1]; ++j) m = kShapes.p[j].dv < m ? kShapes.p[j].dv : m;
@@ -404,8 +409,7 @@ constexpr int shape_dv_max(int R) {
     return m;
 }
 constexpr int shape_slots(int R) {
-    const int n = R < 2 ? 0 : (R < 5 ? 1 : 2);
-    return (kShapes.start[R + 1] - kShapes.start[R]) * (PT_U / (1 << n) + 1) *
+    return (kShapes.start[R + 1] - kShapes.start[R]) * (PT_U / shape_spacing(R) + 1) *
            (PT_V + shape_dv_max(R) - shape_dv_min(R));
 }
 constexpr int adj_max_slots() {
@@ -416,18 +420,23 @@ constexpr int adj_max_slots() {
 constexpr int ADJ_SLOTS = adj_max_slots();
 
 constexpr int ADJ_THREADS = 256;   // block size of the adjoint trace
-constexpr int ADJ_ROUNDS = 3;      // probes per thread and shape, at most
+constexpr int ADJ_ROUNDS = 2;      // probes per thread and shape, at most
 
 template <int R> struct RayBox {
     static constexpr int n = RayAt<R>::n, k = RayAt<R>::k, S = 1 << n;
+    static constexpr int SP = shape_spacing(R), OF = shape_offset(R);
     static constexpr int NP = RayAt<R>::end - RayAt<R>::begin;
     static constexpr int dvlo = shape_dv_min(R), dvhi = shape_dv_max(R);
     static constexpr int NVB = PT_V + dvhi - dvlo;
-    static constexpr int NPROBE = (PT_U / S + 1) * NVB;
+    static constexpr int NPROBE = (PT_U / SP + 1) * NVB;
     static constexpr int ROUNDS = (NPROBE + ADJ_THREADS - 1) / ADJ_THREADS;
     static_assert(dvlo == 0 || dvhi == 0, "a ray is monotone in v");
     static_assert(S <= PT_HALO && dvhi - dvlo <= PT_HALO, "the halo covers every probe of the box");
     static_assert(ROUNDS <= ADJ_ROUNDS, "prefetch registers");
+    static_assert(PT_U % SP == 0 && S <= 2 * SP && SP <= 2 * S, "PT_U / SP + 1 columns cover the box");
+    // first column of the box of a tile at frame column u0 (the smallest
+    // u >= u0 - S with u = OF mod SP)
+    __device__ __forceinline__ static int first(int u0) { return ((u0 - S - OF + SP - 1) & ~(SP - 1)) + OF; }
 };
 
 // dL/dT of the rays of one shape for the thread's probes (round r = probe
@@ -528,15 +537,15 @@ template <int R>
 __device__ __forceinline__ bool adj_probe(const AdjFrame &f, int ua, int i, int &up, int &vp) {
     using B = RayBox<R>;
     const int col = i / B::NVB, vb = i - col * B::NVB;
-    up = ua + col * B::S;
+    up = ua + col * B::SP;
     vp = f.v0 - B::dvhi + vb;
-    return i < B::NPROBE && up >= 1 && up < f.U && vp >= 0 && vp < f.V && t_live(B::n, up >> B::n, B::k);
+    return i < B::NPROBE && up >= 1 && up < f.U && vp >= 0 && vp < f.V;
 }
 
 template <int P, int C, int R>
 __device__ __forceinline__ void adj_prefetch(const Plan &pl, const AdjFrame &f, AdjPre<typename Prec<P>::A, C> &pre) {
     using B = RayBox<R>;
-    const int ua = (f.u0 - 1) & ~(B::S - 1);      // first aligned column >= u0 - S
+    const int ua = B::first(f.u0);
     const GTLevel<P, C> gTl(pl, f.q, B::n);
 #pragma unroll
     for (int r = 0; r < B::ROUNDS; ++r) {
@@ -551,7 +560,7 @@ __device__ __forceinline__ void adj_phase_a(const PairTile<typename Prec<P>::A, 
                                             const AdjPre<typename Prec<P>::A, C> &pre) {
     using A = typename Prec<P>::A;
     using B = RayBox<R>;
-    const int ua = (f.u0 - 1) & ~(B::S - 1);
+    const int ua = B::first(f.u0);
     const int su = f.fwd ? PT_PITCH : -PT_PITCH;
 #pragma unroll
     for (int r = 0; r < B::ROUNDS; ++r) {
@@ -579,8 +588,8 @@ __device__ __forceinline__ void adj_phase_a(const PairTile<typename Prec<P>::A, 
 }
 
 // Phase B for the pieces J .. end-1 of shape R that can reach a pixel whose
-// frame column u has u mod S == RHO (piece J crosses it for the probe at
-// u - du_J only when that column is a probe column, i.e. du_J mod S == RHO):
+// frame column u has u mod SP == RHO (piece J crosses it for the probe at
+// u - du_J only when that column is a probe column, u - du_J = OF mod SP):
 // the selection is made at compile time, so no piece is tested at run time.
 template <class A, int C, int R, int RHO, int J>
 __device__ __forceinline__ void adj_phase_b_res(const AdjSlots<A, C> &sl, int u, int v, int ua, int v0, A (&dE)[C],
@@ -588,8 +597,8 @@ __device__ __forceinline__ void adj_phase_b_res(const AdjSlots<A, C> &sl, int u,
     if constexpr (J < RayAt<R>::end) {
         using B = RayBox<R>;
         using pc = PieceAt<J>;
-        if constexpr ((pc::du & (B::S - 1)) == RHO)
-            sl.add_to((J - RayAt<R>::begin) * B::NPROBE + ((u - pc::du - ua) >> B::n) * B::NVB +
+        if constexpr (((pc::du + B::OF) & (B::SP - 1)) == RHO)
+            sl.add_to((J - RayAt<R>::begin) * B::NPROBE + (u - pc::du - ua) / B::SP * B::NVB +
                           (v - pc::dv - v0 + B::dvhi),
                       dE, dS);
         adj_phase_b_res<A, C, R, RHO, J + 1>(sl, u, v, ua, v0, dE, dS);
@@ -600,8 +609,8 @@ __device__ __forceinline__ void adj_phase_b_res(const AdjSlots<A, C> &sl, int u,
 template <class A, int C, int R, int RHO = 0>
 __device__ __forceinline__ void adj_phase_b(const AdjSlots<A, C> &sl, int u, int v, int ua, int v0, A (&dE)[C],
                                             A &dS) {
-    if constexpr (RHO < RayBox<R>::S) {
-        if ((u & (RayBox<R>::S - 1)) == RHO)
+    if constexpr (RHO < RayBox<R>::SP) {
+        if ((u & (RayBox<R>::SP - 1)) == RHO)
             adj_phase_b_res<A, C, R, RHO, RayAt<R>::begin>(sl, u, v, ua, v0, dE, dS);
         else
             adj_phase_b<A, C, R, RHO + 1>(sl, u, v, ua, v0, dE, dS);
@@ -625,7 +634,7 @@ __device__ __forceinline__ void adj_shapes(const Plan &pl, const PairTile<typena
             if constexpr (R + 1 < HRC_MAXRAY)
                 if (RayAt<R + 1>::n <= nmax) adj_prefetch<P, C, R + 1>(pl, f, pre);
             __syncthreads();
-            const int ua = (f.u0 - 1) & ~(RayBox<R>::S - 1);
+            const int ua = RayBox<R>::first(f.u0);
 #pragma unroll
             for (int i = 0; i < 2; ++i)
                 if (valid[i]) adj_phase_b<A, C, R>(sl, uc[i], v, ua, f.v0, dE[i], dS[i]);
@@ -644,18 +653,29 @@ template <class A, int C> constexpr size_t adj_trace_smem() {
     return PairTile<A, C>::bytes() + (sl > acc ? sl : acc);
 }
 
+// Sums of dL/de ([C][H][W], k = 0) and dL/dsigma ([H][W], k = 1) of frame q
+// (or of the pair beginning with it) when several blocks of one launch share a
+// tile's frames: in the frame's dL/dR_0 and dL/dR_1 buffers, which no later
+// step of the pass reads (they hold at least U V C values each; N >= 2).
+template <class IN> __host__ __device__ inline IN *adj_part(const Plan &pl, int q, int k) {
+    return reinterpret_cast<IN *>(pl.arena + pl.q[q].gRoff[k]);
+}
+
 // dL/de and dL/dsigma of quadrant pair `pair` for one tile.  Each thread
 // owns two pixels of the tile (columns c[i] along u, its lane along v) and
 // accumulates them in registers over both frames of the pair.  Pair 0
-// writes the image gradients, pair 1 (launched after it) adds to them.
+// writes the image gradients, pair 1 (launched after it) adds to them, or
+// both go to planes that k_adj_combine sums.
 // With tme / tms (fp32 inputs) the tile region is fetched by TMA tensor
 // copies; a copy wait that gives up records its code in the plan's status
 // word and leaves the tile's gradients unwritten.
+// fmask: the pair's frames to take (bits 0, 1); add: add to ge / gs (pair 1
+// launched after pair 0) instead of writing them.
 template <int P, int C, class IN>
 __device__ __forceinline__ void body_adj_trace(const Plan &pl, const IN *__restrict__ e, const IN *__restrict__ s,
                                                IN *__restrict__ ge, IN *__restrict__ gs, int pair, int bx, int by,
                                                unsigned char *smem, const CUtensorMap *tme = nullptr,
-                                               const CUtensorMap *tms = nullptr) {
+                                               const CUtensorMap *tms = nullptr, int fmask = 3, bool add = false) {
     using A = typename Prec<P>::A;
     PairTile<A, C> tt(smem);
     const AdjSlots<A, C> sl{reinterpret_cast<A *>(smem + PairTile<A, C>::bytes())};
@@ -694,7 +714,7 @@ __device__ __forceinline__ void body_adj_trace(const Plan &pl, const IN *__restr
     for (int qq = 0; qq < 2; ++qq) {
         const int q = 2 * pair + qq;
         const QuadGeom &g = pl.q[q];
-        if (g.N < 1) continue;
+        if (g.N < 1 || !((fmask >> qq) & 1)) continue;
         AdjFrame f;
         f.q = q;
         f.U = g.U;
@@ -728,8 +748,8 @@ __device__ __forceinline__ void body_adj_trace(const Plan &pl, const IN *__restr
             acc[(C * PT_V + lane) * (PT_U + 1) + c] = dS[i];
         } else {
 #pragma unroll
-            for (int k = 0; k < C; ++k) ge[k * HW + pix] = IN(A(ge[k * HW + pix]) + dE[i][k]);
-            gs[pix] = IN(A(gs[pix]) + dS[i]);
+            for (int k = 0; k < C; ++k) ge[k * HW + pix] = IN(add ? A(ge[k * HW + pix]) + dE[i][k] : dE[i][k]);
+            gs[pix] = IN(add ? A(gs[pix]) + dS[i] : dS[i]);
         }
     }
     if (pair == 0) {

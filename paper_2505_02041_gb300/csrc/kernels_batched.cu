@@ -100,7 +100,7 @@ __global__ void __launch_bounds__(256, KIND == 1 ? 3 : 2) k_batched_tiles(BatchA
         body_trace012<P, C>(pl, (const float *)e, (const float *)s, (const double *)e, (const double *)s, 15, bx, by,
                             smem);
     else
-        body_adj_trace<P, C, IN>(pl, e, s, (IN *)a.ge + eo, (IN *)a.gs + so, pair, bx, by, smem);
+        body_adj_trace<P, C, IN>(pl, e, s, (IN *)a.ge + eo, (IN *)a.gs + so, pair, bx, by, smem, nullptr, nullptr, 3, pair == 1);
 }
 
 // The merge cascade of every scene.  MODE 0: the forward's merge and

@@ -52,7 +52,54 @@ __global__ void __launch_bounds__(ADJ_THREADS, 3) k_adj_trace(Plan pl, const IN 
                                                    const __grid_constant__ CUtensorMap tms, int use_tma) {
     extern __shared__ __align__(128) unsigned char tb_smem[];
     body_adj_trace<P, C, IN>(pl, e, s, ge, gs, pair, blockIdx.x, blockIdx.y, tb_smem, use_tma ? &tme : nullptr,
-                             use_tma ? &tms : nullptr);
+                             use_tma ? &tms : nullptr, 3, pair == 1);
+}
+
+// Both pairs' adjoint traces in one launch.  FB = 2: block b < n0 takes tile b
+// of pair 0 (into ge / gs), the others pair 1 (into the planes of frame 2).
+// FB = 1: every frame its own blocks and planes, frames 0 .. 3 in order.
+// k_adj_combine adds the planes.
+template <int P, int C, class IN, int FB>
+__global__ void __launch_bounds__(ADJ_THREADS, 3) k_adj_trace_all(Plan pl, const IN *__restrict__ e,
+                                                                  const IN *__restrict__ s, IN *ge, IN *gs, int n0, int n1,
+                                                                  int nx0, int nx1, const __grid_constant__ CUtensorMap me0,
+                                                                  const __grid_constant__ CUtensorMap ms0,
+                                                                  const __grid_constant__ CUtensorMap me1,
+                                                                  const __grid_constant__ CUtensorMap ms1, int use_tma) {
+    extern __shared__ __align__(128) unsigned char tb_smem[];
+    constexpr int BF = 2 / FB;                            // blocks per tile
+    const int b = (int)blockIdx.x, pair = b >= BF * n0, r = pair ? b - BF * n0 : b, nt = pair ? n1 : n0;
+    const int half = FB == 1 && r >= nt, t = half ? r - nt : r, nx = pair ? nx1 : nx0, q = 2 * pair + half;
+    if (FB == 1 || pair) {
+        ge = adj_part<IN>(pl, q, 0);
+        gs = adj_part<IN>(pl, q, 1);
+    }
+    body_adj_trace<P, C, IN>(pl, e, s, ge, gs, pair, t % nx, t / nx, tb_smem, use_tma ? (pair ? &me1 : &me0) : nullptr,
+                             use_tma ? (pair ? &ms1 : &ms0) : nullptr, FB == 2 ? 3 : 1 << half);
+}
+
+// dL/de and dL/dsigma from the planes of k_adj_trace_all: (q0 + q1) + (q2 + q3).
+template <int C, class IN, int FB>
+__global__ void __launch_bounds__(256) k_adj_combine(Plan pl, IN *__restrict__ ge, IN *__restrict__ gs) {
+    const long long HW = (long long)pl.W * pl.H, n = (C + 1) * HW;
+    const IN *pe[4], *ps[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        pe[q] = adj_part<IN>(pl, q, 0);
+        ps[q] = adj_part<IN>(pl, q, 1) - C * HW;
+    }
+    for (long long i = blockIdx.x * 256LL + threadIdx.x; i < n; i += gridDim.x * 256LL) {
+        const bool es = i < C * HW;
+        IN *o = (es ? ge : gs - C * HW) + i;
+        if constexpr (FB == 2) {
+            *o += (es ? pe[2] : ps[2])[i];
+        } else {
+            IN v[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) v[q] = (es ? pe[q] : ps[q])[i];
+            *o = (v[0] + v[1]) + (v[2] + v[3]);
+        }
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -102,8 +149,11 @@ static cudaError_t bwd_impl(const Plan &pl, const RayTable &rt, const void *e, c
     using IN = typename std::conditional<P == P_FP64, double, float>::type;
     const int mt = pl.mthreads, ts = 2 * mt > 512 ? 512 : 2 * mt;   // paired-v / single-v block sizes
     const bool env = plan_has_env(pl);   // kernels compiled for an environment map
-    int Nmax = 0;
-    for (int q = 0; q < 4; ++q) Nmax = pl.q[q].N > Nmax ? pl.q[q].N : Nmax;
+    int Nmax = 0, Nmin = pl.q[0].N;
+    for (int q = 0; q < 4; ++q) {
+        Nmax = pl.q[q].N > Nmax ? pl.q[q].N : Nmax;
+        Nmin = pl.q[q].N < Nmin ? pl.q[q].N : Nmin;
+    }
     const double ab = P == P_FP64 ? 8.0 : 4.0;
     const double img = double(pl.W) * pl.H;
     // live columns x >= 1 only (column 0 is dead)
@@ -179,7 +229,45 @@ static cudaError_t bwd_impl(const Plan &pl, const RayTable &rt, const void *e, c
     {
         using A = typename Prec<P>::A;
         const size_t smem = adj_trace_smem<A, C>();
-        for (int pair = 0; pair < 2; ++pair) {
+        const int nx0 = pair_tiles_x(0, pl.W), nx1 = pair_tiles_x(1, pl.W);
+        const int n0 = nx0 * pair_tiles_y(0, pl.H), n1 = nx1 * pair_tiles_y(1, pl.H);
+        // Both pairs in one launch and their sum in a second one: two launches
+        // of 4.5 waves each (1024^2, 456 blocks resident) become one of 9, and
+        // pair 1 no longer reads what pair 0 wrote.  While a block per tile and
+        // frame fits the GPU at once (3 blocks per SM: 2 (n0 + n1) <= 456), a
+        // tile's two frames are halved too.  Adjoint trace in all, C = 3, fp32,
+        // us, one pair after the other / pairs at once / frames at once:
+        // 64^2 40.9 / 24.4 / 17.3, 256^2 44.0 / 30.2 / 35.9, 512^2 97 / 79 / 85,
+        // 1024^2 269 / 254 / 309, 2048^2 987 / 966 / 1216.  The planes need
+        // dL/dR_1 buffers (N >= 2 in every frame).
+        const bool all = Nmin >= 2;
+        if (all) {
+            const bool one = pl.solo && n0 + n1 <= 228;   // a frame per block
+            double by = img * (pl.C + 1) * ab * (one ? 10.0 : 5.0);   // the inputs, the planes written and read, the sums
+            for (int q = 0; q < 4; ++q)
+                for (int n = 0; n <= 2; ++n) by += gTbytes(q, n);
+            rec->begin(K_ADJ_TRACE, 0, by);
+            CUtensorMap m[4];
+            std::memset(m, 0, sizeof(m));
+            const int use_tma = (P != P_FP64 && encode_image_maps(pl, e, s, PT_RU, PT_RV, m[0], m[1]) &&
+                                 encode_image_maps(pl, e, s, PT_RV, PT_RU, m[2], m[3])) ? 1 : 0;
+            const IN *ei = (const IN *)e, *si = (const IN *)s;
+            IN *geo = (IN *)ge, *gso = (IN *)gs;
+            const long long nb = ((long long)(pl.C + 1) * pl.W * pl.H + 255) / 256;
+            const unsigned cb = (unsigned)(nb < 2432 ? nb : 2432);
+            if (one) {
+                k_adj_trace_all<P, C, IN, 1><<<2 * (n0 + n1), ADJ_THREADS, smem, st>>>(pl, ei, si, geo, gso, n0, n1, nx0, nx1,
+                                                                                    m[0], m[1], m[2], m[3], use_tma);
+                k_adj_combine<C, IN, 1><<<cb, 256, 0, st>>>(pl, geo, gso);
+            } else {
+                k_adj_trace_all<P, C, IN, 2><<<n0 + n1, ADJ_THREADS, smem, st>>>(pl, ei, si, geo, gso, n0, n1, nx0, nx1, m[0],
+                                                                              m[1], m[2], m[3], use_tma);
+                k_adj_combine<C, IN, 2><<<cb, 256, 0, st>>>(pl, geo, gso);
+            }
+            rec->end();
+            *launches += 2;
+        }
+        for (int pair = 0; pair < 2 && !all; ++pair) {
             double by = img * (pl.C + 1) * ab * (pair == 0 ? 1.0 : 2.0);   // pair 1 adds to the gradients
             for (int q = 2 * pair; q < 2 * pair + 2; ++q)
                 for (int n = 0; n <= 2; ++n) by += gTbytes(q, n);
@@ -220,9 +308,17 @@ static cudaError_t prepare_bwd_prec() {
         if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
     };
     set((const void *)k_adj_trace<P, 1, IN>, adj_trace_smem<A, 1>());
+    set((const void *)k_adj_trace_all<P, 1, IN, 1>, adj_trace_smem<A, 1>());
+    set((const void *)k_adj_trace_all<P, 1, IN, 2>, adj_trace_smem<A, 1>());
     set((const void *)k_adj_trace<P, 2, IN>, adj_trace_smem<A, 2>());
+    set((const void *)k_adj_trace_all<P, 2, IN, 1>, adj_trace_smem<A, 2>());
+    set((const void *)k_adj_trace_all<P, 2, IN, 2>, adj_trace_smem<A, 2>());
     set((const void *)k_adj_trace<P, 3, IN>, adj_trace_smem<A, 3>());
+    set((const void *)k_adj_trace_all<P, 3, IN, 1>, adj_trace_smem<A, 3>());
+    set((const void *)k_adj_trace_all<P, 3, IN, 2>, adj_trace_smem<A, 3>());
     set((const void *)k_adj_trace<P, 4, IN>, adj_trace_smem<A, 4>());
+    set((const void *)k_adj_trace_all<P, 4, IN, 1>, adj_trace_smem<A, 4>());
+    set((const void *)k_adj_trace_all<P, 4, IN, 2>, adj_trace_smem<A, 4>());
     return e;
 }
 

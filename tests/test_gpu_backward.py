@@ -188,3 +188,24 @@ def test_backward_recompute_mode(W, H, C, seed):
     _lib.hrc_fluence_backward(h.ctx, gd, ge2, gs2)
     ge_r2, gs_r2 = oracle.fluence_adjoint(e, s * np.float32(1.7), gF)
     assert err_max(ge2.cpu().numpy(), ge_r2) <= 1e-4 and err_max(gs2.cpu().numpy(), gs_r2) <= 1e-4
+
+
+@pytest.mark.parametrize("W,H,C,casc,seed", [
+    (3, 2, 1, 0, 50), (3, 3, 2, 0, 51), (4, 70, 3, 1, 52), (70, 5, 1, 2, 53), (335, 341, 1, 0, 54), (352, 352, 3, 0, 55),
+    (17, 33, 4, 0, 56), (480, 250, 2, 0, 57),
+])
+def test_adjoint_trace_forms(W, H, C, casc, seed):
+    """The adjoint trace in its three forms -- one pair after the other (a
+    frame with fewer than two cascades), a frame per block (few tiles), a pair
+    per block -- on either side of the lines between them, with odd extents:
+    fp32 against the oracle, and in fp64 to rounding."""
+    require_gpu()
+    e, s = scenes.random_scene(W, H, C, seed)
+    gF = scenes.rng(3000 + seed).normal(size=e.shape)
+    ge_r, gs_r = oracle.fluence_adjoint(e, s, gF.astype(np.float32), casc)
+    ge, gs = _gpu_grads(e, s, gF.astype(np.float32), "fp32", casc)
+    assert err_max(ge, ge_r) <= 1e-4 and err_max(gs, gs_r) <= 1e-4
+    if W * H < 20000:
+        ge_r, gs_r = oracle.fluence_adjoint(e, s, gF, casc)
+        ge, gs = _gpu_grads(e.astype(np.float64), s.astype(np.float64), gF, "fp64", casc)
+        assert err_max(ge, ge_r) <= 1e-10 and err_max(gs, gs_r) <= 1e-10
