@@ -465,23 +465,6 @@ __device__ __forceinline__ void merge_down_entry(const Plan &pl, int q, int n, i
         // four consecutive v (v a multiple of 4, n >= 1): one 4-wide access
         // per plane and row; a far run whose even offset is not a multiple
         // of 4, or that crosses the grid edge, is read as two pairs
-        auto loadR4 = [&](const RLevel<P, C> &R1, int xr, int j, int c, int vq, A (&r)[4]) {
-            if ((vq & 3) == 0 && vq >= 0 && vq + 3 < g.V) {
-                R1.load4(xr, j, c, vq, r);
-                return;
-            }
-            const A ev = renv<P, C, ENV>(pl, q, n + 1, j, c);
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const int vp = vq + 2 * h;
-                if (vp >= 0 && vp < g.V) {
-                    R1.load2(xr, j, c, vp, r[2 * h], r[2 * h + 1]);
-                    if (vp + 1 >= g.V) r[2 * h + 1] = ev;
-                } else {
-                    r[2 * h] = r[2 * h + 1] = ev;
-                }
-            }
-        };
         if (x & 1) {   // Eq. 14
             TLevel<P, C> Tn(pl, q, n);
             const int xq = (x + 1) >> 1;
@@ -494,15 +477,14 @@ __device__ __forceinline__ void merge_down_entry(const Plan &pl, int q, int n, i
                 const A Aj = sg == 0 ? Ap : Am;
                 Iv<P, C> t[4];
                 Tn.load4(x, kk, v, t);
-                const int vq = v + 2 * kk - s;
+                A r[C][4], ev[C];
 #pragma unroll
-                for (int c = 0; c < C; ++c) {
-                    A r[4];
-                    if (rq_ok) loadR4(R1, xq, j, c, vq, r);
-                    else r[0] = r[1] = r[2] = r[3] = renv<P, C, ENV>(pl, q, n + 1, j, c);
+                for (int c = 0; c < C; ++c) ev[c] = renv<P, C, ENV>(pl, q, n + 1, j, c);
+                rows4<C>(rq_ok, R1.base + R1.idx(rq_ok ? xq : 0, rq_ok ? j : 0, 0, 0), g.Vs, v + 2 * kk - s, g.V, ev, r);
 #pragma unroll
-                    for (int l = 0; l < 4; ++l) acc[l][c] += fma(Aj, t[l].L[c], t[l].trans() * r[l]);
-                }
+                for (int c = 0; c < C; ++c)
+#pragma unroll
+                    for (int l = 0; l < 4; ++l) acc[l][c] += fma(Aj, t[l].L[c], t[l].trans() * r[c][l]);
             }
         } else {       // Eqs. 15-17
             TLevel<P, C> T1(pl, q, n + 1);
@@ -516,19 +498,22 @@ __device__ __forceinline__ void merge_down_entry(const Plan &pl, int q, int n, i
                 const A Aj = sg == 0 ? Ap : Am;
                 Iv<P, C> t[4];
                 T1.load4(x2, kk, v, t);
-                const int vq = v + 2 * kk - 2 * s;
+                A r0[C][4], r1[C][4], ev[C];
 #pragma unroll
-                for (int c = 0; c < C; ++c) {
-                    A r0[4], r1[4];
-                    const A ev = renv<P, C, ENV>(pl, q, n + 1, j, c);
-                    if (!top) R1.load4(x2, j, c, v, r0);
-                    else r0[0] = r0[1] = r0[2] = r0[3] = ev;
-                    if (r1_ok) loadR4(R1, x2 + 1, j, c, vq, r1);
-                    else r1[0] = r1[1] = r1[2] = r1[3] = ev;
+                for (int c = 0; c < C; ++c) ev[c] = renv<P, C, ENV>(pl, q, n + 1, j, c);
+                if (!top) {
+#pragma unroll
+                    for (int c = 0; c < C; ++c) R1.load4(x2, j, c, v, r0[c]);
+                } else {
+#pragma unroll
+                    for (int c = 0; c < C; ++c) r0[c][0] = r0[c][1] = r0[c][2] = r0[c][3] = ev[c];
+                }
+                rows4<C>(r1_ok, R1.base + R1.idx(r1_ok ? x2 + 1 : 0, r1_ok ? j : 0, 0, 0), g.Vs, v + 2 * kk - 2 * s, g.V, ev, r1);
+#pragma unroll
+                for (int c = 0; c < C; ++c)
 #pragma unroll
                     for (int l = 0; l < 4; ++l)
-                        acc[l][c] += A(0.5) * (r0[l] + fma(Aj, t[l].L[c], t[l].trans() * r1[l]));
-                }
+                        acc[l][c] += A(0.5) * (r0[c][l] + fma(Aj, t[l].L[c], t[l].trans() * r1[c][l]));
             }
         }
         return;
@@ -839,22 +824,25 @@ __device__ __forceinline__ void r0_pair_add(const Plan &pl, int q, int x, int v,
             T0.load2_ef(x, j, v, pol, t0, t1);
             const A tr0 = t0.trans(), tr1 = t1.trans();
             const int vq = v + 2 * j - 1;       // odd
+            A r0[C], r1[C], other;              // each range tested once for all channels (see rows4)
+            if (rq_ok && vq >= 0 && vq < g.V) {
+#pragma unroll
+                for (int c = 0; c < C; ++c) R1.load2(xq, j, c, vq - 1, other, r0[c]);
+            } else {
+#pragma unroll
+                for (int c = 0; c < C; ++c) r0[c] = renv<P, C, ENV>(pl, q, 1, j, c);
+            }
+            if (rq_ok && vq + 1 < g.V) {
+#pragma unroll
+                for (int c = 0; c < C; ++c) R1.load2(xq, j, c, vq + 1, r1[c], other);
+            } else {
+#pragma unroll
+                for (int c = 0; c < C; ++c) r1[c] = renv<P, C, ENV>(pl, q, 1, j, c);
+            }
 #pragma unroll
             for (int c = 0; c < C; ++c) {
-                const A ev = renv<P, C, ENV>(pl, q, 1, j, c);
-                A r0 = ev, r1 = ev, lo, hi;
-                if (rq_ok) {
-                    if (vq >= 0 && vq < g.V) {
-                        R1.load2(xq, j, c, vq - 1, lo, hi);
-                        r0 = hi;
-                    }
-                    if (vq + 1 < g.V) {
-                        R1.load2(xq, j, c, vq + 1, lo, hi);
-                        r1 = lo;
-                    }
-                }
-                acc[0][c] += fma(Aj, t0.L[c], tr0 * r0);
-                acc[1][c] += fma(Aj, t1.L[c], tr1 * r1);
+                acc[0][c] += fma(Aj, t0.L[c], tr0 * r0[c]);
+                acc[1][c] += fma(Aj, t1.L[c], tr1 * r1[c]);
             }
         }
     } else {                                    // Eqs. 15-17 at n = 0: k = 2, 0 and j = 1, 0
@@ -869,17 +857,29 @@ __device__ __forceinline__ void r0_pair_add(const Plan &pl, int q, int x, int v,
             T1.load2_ef(x2, 2 * j, v, pol, t0, t1);
             const A tr0 = t0.trans(), tr1 = t1.trans();
             const int vq = v + 4 * j - 2;       // even
+            A n0[C], n1[C], f0[C], f1[C];
+            if (!top) {
+#pragma unroll
+                for (int c = 0; c < C; ++c) R1.load2(x2, j, c, v, n0[c], n1[c]);
+            } else {
+#pragma unroll
+                for (int c = 0; c < C; ++c) n0[c] = n1[c] = renv<P, C, ENV>(pl, q, 1, j, c);
+            }
+            if (r1_ok && vq >= 0 && vq < g.V) {
+#pragma unroll
+                for (int c = 0; c < C; ++c) R1.load2(x2 + 1, j, c, vq, f0[c], f1[c]);
+                if (vq + 1 >= g.V) {
+#pragma unroll
+                    for (int c = 0; c < C; ++c) f1[c] = renv<P, C, ENV>(pl, q, 1, j, c);
+                }
+            } else {
+#pragma unroll
+                for (int c = 0; c < C; ++c) f0[c] = f1[c] = renv<P, C, ENV>(pl, q, 1, j, c);
+            }
 #pragma unroll
             for (int c = 0; c < C; ++c) {
-                const A ev = renv<P, C, ENV>(pl, q, 1, j, c);
-                A n0 = ev, n1 = ev, f0 = ev, f1 = ev;
-                if (!top) R1.load2(x2, j, c, v, n0, n1);
-                if (r1_ok && vq >= 0 && vq < g.V) {
-                    R1.load2(x2 + 1, j, c, vq, f0, f1);
-                    if (vq + 1 >= g.V) f1 = ev;
-                }
-                acc[0][c] += A(0.5) * (n0 + fma(Aj, t0.L[c], tr0 * f0));
-                acc[1][c] += A(0.5) * (n1 + fma(Aj, t1.L[c], tr1 * f1));
+                acc[0][c] += A(0.5) * (n0[c] + fma(Aj, t0.L[c], tr0 * f0[c]));
+                acc[1][c] += A(0.5) * (n1[c] + fma(Aj, t1.L[c], tr1 * f1[c]));
             }
         }
     }
@@ -1006,25 +1006,32 @@ __device__ __forceinline__ void r0_quad_add(const Plan &pl, int q, int x, int v,
             A tr[4];
 #pragma unroll
             for (int l = 0; l < 4; ++l) tr[l] = t[l].trans();
+            // far run v + 2j - 1 .. v + 2j + 2: the quad at v and the entry
+            // before or after it (each range tested once for all channels)
+            A w[C][4], b[C];
 #pragma unroll
-            for (int c = 0; c < C; ++c) {
-                const A ev = renv<P, C, ENV>(pl, q, 1, j, c);
-                A r[4] = {ev, ev, ev, ev}, w[4];
-                if (rq_ok) {
-                    // far run v + 2j - 1 .. v + 2j + 2: the quad at v and the entry before or after it
-                    R1.load4(xq, j, c, v, w);
-                    if (j) {
+            for (int c = 0; c < C; ++c) b[c] = renv<P, C, ENV>(pl, q, 1, j, c);
+            if (rq_ok) {
 #pragma unroll
-                        for (int l = 0; l < 3; ++l)
-                            if (v + 1 + l < V) r[l] = w[l + 1];
-                        if (v + 4 < V) r[3] = R1.load(xq, j, c, v + 4);
-                    } else {
-                        if (v >= 1) r[0] = R1.load(xq, j, c, v - 1);
+                for (int c = 0; c < C; ++c) R1.load4(xq, j, c, v, w[c]);
+                if (j ? v + 4 < V : v >= 1) {
+#pragma unroll
+                    for (int c = 0; c < C; ++c) b[c] = R1.load(xq, j, c, j ? v + 4 : v - 1);
+                }
+                if (v + 3 >= V) {
+#pragma unroll
+                    for (int c = 0; c < C; ++c)
 #pragma unroll
                         for (int l = 1; l < 4; ++l)
-                            if (v + l - 1 < V) r[l] = w[l - 1];
-                    }
+                            if (v + l >= V) w[c][l] = renv<P, C, ENV>(pl, q, 1, j, c);
                 }
+            } else {
+#pragma unroll
+                for (int c = 0; c < C; ++c) w[c][0] = w[c][1] = w[c][2] = w[c][3] = b[c];
+            }
+#pragma unroll
+            for (int c = 0; c < C; ++c) {
+                const A r[4] = {j ? w[c][1] : b[c], j ? w[c][2] : w[c][0], j ? w[c][3] : w[c][1], j ? b[c] : w[c][2]};
 #pragma unroll
                 for (int l = 0; l < 4; ++l) acc[l][c] += fma(Aj, t[l].L[c], tr[l] * r[l]);
             }
@@ -1042,31 +1049,44 @@ __device__ __forceinline__ void r0_quad_add(const Plan &pl, int q, int x, int v,
             A tr[4];
 #pragma unroll
             for (int l = 0; l < 4; ++l) tr[l] = t[l].trans();
+            // far run v + 4j - 2 .. v + 4j + 1: the quad at v and the pair
+            // before or after it
+            A nr[C][4], w[C][4], b0[C], b1[C];
 #pragma unroll
-            for (int c = 0; c < C; ++c) {
-                const A ev = renv<P, C, ENV>(pl, q, 1, j, c);
-                A n0[4] = {ev, ev, ev, ev}, f[4] = {ev, ev, ev, ev}, w[4];
-                if (!top) R1.load4(x2, j, c, v, n0);
-                if (r1_ok) {
-                    // far run v + 4j - 2 .. v + 4j + 1: the quad at v and the pair after or before it
-                    R1.load4(x2 + 1, j, c, v, w);
-                    if (j) {
-                        if (v + 2 < V) f[0] = w[2];
-                        if (v + 3 < V) f[1] = w[3];
-                        if (v + 4 < V) {
-                            A p0, p1;
-                            R1.load2(x2 + 1, j, c, v + 4, p0, p1);
-                            f[2] = p0;
-                            if (v + 5 < V) f[3] = p1;
-                        }
-                    } else {
-                        if (v >= 2) R1.load2(x2 + 1, j, c, v - 2, f[0], f[1]);
-                        if (v < V) f[2] = w[0];
-                        if (v + 1 < V) f[3] = w[1];
+            for (int c = 0; c < C; ++c) b0[c] = b1[c] = renv<P, C, ENV>(pl, q, 1, j, c);
+            if (!top) {
+#pragma unroll
+                for (int c = 0; c < C; ++c) R1.load4(x2, j, c, v, nr[c]);
+            } else {
+#pragma unroll
+                for (int c = 0; c < C; ++c) nr[c][0] = nr[c][1] = nr[c][2] = nr[c][3] = b0[c];
+            }
+            if (r1_ok) {
+#pragma unroll
+                for (int c = 0; c < C; ++c) R1.load4(x2 + 1, j, c, v, w[c]);
+                if (j ? v + 4 < V : v >= 2) {
+#pragma unroll
+                    for (int c = 0; c < C; ++c) R1.load2(x2 + 1, j, c, j ? v + 4 : v - 2, b0[c], b1[c]);
+                }
+                if (v + 5 >= V) {
+#pragma unroll
+                    for (int c = 0; c < C; ++c) {
+                        const A ev = renv<P, C, ENV>(pl, q, 1, j, c);
+                        if (j) b1[c] = ev;
+#pragma unroll
+                        for (int l = 1; l < 4; ++l)
+                            if (v + l >= V) w[c][l] = ev;
                     }
                 }
+            } else {
 #pragma unroll
-                for (int l = 0; l < 4; ++l) acc[l][c] += A(0.5) * (n0[l] + fma(Aj, t[l].L[c], tr[l] * f[l]));
+                for (int c = 0; c < C; ++c) w[c][0] = w[c][1] = w[c][2] = w[c][3] = b0[c];
+            }
+#pragma unroll
+            for (int c = 0; c < C; ++c) {
+                const A f[4] = {j ? w[c][2] : b0[c], j ? w[c][3] : b1[c], j ? b0[c] : w[c][0], j ? b1[c] : w[c][1]};
+#pragma unroll
+                for (int l = 0; l < 4; ++l) acc[l][c] += A(0.5) * (nr[c][l] + fma(Aj, t[l].L[c], tr[l] * f[l]));
             }
         }
     }

@@ -291,6 +291,35 @@ __device__ __forceinline__ void st4(__nv_bfloat16 *p, const float (&r)[4]) {
     *reinterpret_cast<uint2 *>(p) = u;
 }
 
+// Entries v .. v + 3 (v even) of NC rows of V entries, `stride` apart; those
+// outside [0, V), and all of them without `ok`, are ev[c].  4-wide loads where
+// v is a multiple of 4 and the four lie inside, else pairs.  The range is
+// tested once for all rows: a test per row puts every row's load behind a
+// branch of its own, and the rows are then waited for one after another.
+template <int NC, class S, class A>
+__device__ __forceinline__ void rows4(bool ok, const S *row, int stride, int v, int V, const A (&ev)[NC],
+                                      A (&r)[NC][4]) {
+    if (ok && (v & 3) == 0 && v >= 0 && v + 3 < V) {
+#pragma unroll
+        for (int c = 0; c < NC; ++c) ld4(row + (long long)c * stride + v, r[c]);
+        return;
+    }
+#pragma unroll
+    for (int h = 0; h < 4; h += 2) {
+        if (ok && v + h >= 0 && v + h < V) {
+#pragma unroll
+            for (int c = 0; c < NC; ++c) ld2(row + (long long)c * stride + v + h, r[c][h], r[c][h + 1]);
+            if (v + h + 1 >= V) {
+#pragma unroll
+                for (int c = 0; c < NC; ++c) r[c][h + 1] = ev[c];
+            }
+        } else {
+#pragma unroll
+            for (int c = 0; c < NC; ++c) r[c][h] = r[c][h + 1] = ev[c];
+        }
+    }
+}
+
 // ---------------------------------------------------------------------------
 // L2 residency.  The merge down reads each T row from HBM (the merge up
 // wrote it long before), while R_{n+1} -- written by the previous launch --
