@@ -96,6 +96,79 @@ template <class A, int E> struct Lanes {
     A x[E];
 };
 
+// As rows4, for the transmittance of a T row together with NG adjoint planes:
+// t = the transmittance at v .. v + 3 and r[c] = gr[c Vs + v ..], vacuum and
+// zero outside.
+template <int P, int C, int NG>
+__device__ __forceinline__ void shifted4(bool ok, const char *trow, const typename Prec<P>::A *gr, int Vs, int v, int V,
+                                         typename Prec<P>::A (&t)[4], typename Prec<P>::A (&r)[NG][4]) {
+    using A = typename Prec<P>::A;
+    using ST = typename Prec<P>::ST;
+    const ST *tp = reinterpret_cast<const ST *>(trow + (size_t)C * Vs * sizeof(typename Prec<P>::SL));
+    const A vac = Prec<P>::LOG ? A(0) : A(1);
+    if (ok && (v & 3) == 0 && v >= 0 && v + 3 < V) {
+        ld4(tp + v, t);
+#pragma unroll
+        for (int c = 0; c < NG; ++c) ld4(gr + (long long)c * Vs + v, r[c]);
+    } else {
+#pragma unroll
+        for (int h = 0; h < 4; h += 2) {
+            t[h] = t[h + 1] = vac;
+#pragma unroll
+            for (int c = 0; c < NG; ++c) r[c][h] = r[c][h + 1] = A(0);
+            if (ok && v + h >= 0 && v + h < V) {
+                ld2(tp + v + h, t[h], t[h + 1]);
+#pragma unroll
+                for (int c = 0; c < NG; ++c) ld2(gr + (long long)c * Vs + v + h, r[c][h], r[c][h + 1]);
+                if (v + h + 1 >= V) {
+                    t[h + 1] = vac;
+#pragma unroll
+                    for (int c = 0; c < NG; ++c) r[c][h + 1] = A(0);
+                }
+            }
+        }
+    }
+#pragma unroll
+    for (int l = 0; l < 4; ++l) t[l] = Prec<P>::LOG ? fexp(-t[l]) : t[l];
+}
+
+// The interval of a T row at v .. v + 3 (vacuum outside): radiances and
+// linear transmittance.
+template <int P, int C>
+__device__ __forceinline__ void interval4(bool ok, const char *trow, int Vs, int v, int V, typename Prec<P>::A (&L)[C][4],
+                                          typename Prec<P>::A (&t)[4]) {
+    using A = typename Prec<P>::A;
+    using SL = typename Prec<P>::SL;
+    using ST = typename Prec<P>::ST;
+    const SL *lp = reinterpret_cast<const SL *>(trow);
+    const ST *tp = reinterpret_cast<const ST *>(trow + (size_t)C * Vs * sizeof(SL));
+    const A vac = Prec<P>::LOG ? A(0) : A(1);
+    if (ok && (v & 3) == 0 && v >= 0 && v + 3 < V) {
+        ld4(tp + v, t);
+#pragma unroll
+        for (int c = 0; c < C; ++c) ld4(lp + (long long)c * Vs + v, L[c]);
+    } else {
+#pragma unroll
+        for (int h = 0; h < 4; h += 2) {
+            t[h] = t[h + 1] = vac;
+#pragma unroll
+            for (int c = 0; c < C; ++c) L[c][h] = L[c][h + 1] = A(0);
+            if (ok && v + h >= 0 && v + h < V) {
+                ld2(tp + v + h, t[h], t[h + 1]);
+#pragma unroll
+                for (int c = 0; c < C; ++c) ld2(lp + (long long)c * Vs + v + h, L[c][h], L[c][h + 1]);
+                if (v + h + 1 >= V) {
+                    t[h + 1] = vac;
+#pragma unroll
+                    for (int c = 0; c < C; ++c) L[c][h + 1] = A(0);
+                }
+            }
+        }
+    }
+#pragma unroll
+    for (int l = 0; l < 4; ++l) t[l] = Prec<P>::LOG ? fexp(-t[l]) : t[l];
+}
+
 // ---------------------------------------------------------------------------
 // dL/dR_{n+1}(x', j, w).  For cone index j (j + 1/2 at level n+1) the parent
 // cone at level n is ip = j >> 1 and its edge direction kk = (j + 1) >> 1
@@ -165,6 +238,51 @@ __device__ __forceinline__ void body_adj_R(const Plan &pl, const RowSplitB &rs, 
         if (E == 2) gR1.store2(x1, j, c, w, acc[0][c], acc[E - 1][c]);
         else gR1.store(x1, j, c, w, acc[0][c]);
     }
+}
+
+// body_adj_R with four consecutive w per thread (n >= 1: every shift even).
+template <int P, int C>
+__device__ __forceinline__ void body_adj_R4(const Plan &pl, const RowSplitB &rs, int n, long long bx, int by) {
+    using A = typename Prec<P>::A;
+    int local;
+    const int q = quadrant_of(rs, bx, local);   // row = (q, x', j) at level n+1, x' >= 1
+    const QuadGeom &g = pl.q[q];
+    const int w = 4 * (by * blockDim.x + threadIdx.x), V = g.V, Vs = g.Vs;
+    if (w >= V) return;
+    local += 2 << n;
+    const int x1 = local >> (n + 1), j = local & ((2 << n) - 1);
+    const int ip = j >> 1, kk = (j + 1) >> 1;
+    const int d = 2 * kk - (1 << n);
+    const GRLevel<P, C> gRn(pl, q, n), gR1(pl, q, n + 1);
+    A acc[C][4];
+#pragma unroll
+    for (int c = 0; c < C; ++c)
+#pragma unroll
+        for (int l = 0; l < 4; ++l) acc[c][l] = A(0);
+    // + weight T(xt, kt) gR_n(xp, ip) at w - sh
+    auto term = [&](int xp, int sh, A wgt, const char *trow) {
+        A t[4] = {wgt, wgt, wgt, wgt}, r[C][4];
+        const A *gr = gRn.base + gRn.idx(xp, ip, 0, 0);
+        if (trow) {
+            shifted4<P, C, C>(true, trow, gr, Vs, w - sh, V, t, r);
+#pragma unroll
+            for (int l = 0; l < 4; ++l) t[l] *= wgt;
+        } else {
+#pragma unroll
+            for (int c = 0; c < C; ++c) ld4(gr + c * Vs + w, r[c]);      // the term without a shift
+        }
+#pragma unroll
+        for (int c = 0; c < C; ++c)
+#pragma unroll
+            for (int l = 0; l < 4; ++l) acc[c][l] = fma(t[l], r[c][l], acc[c][l]);
+    };
+    const int xo = 2 * x1 - 1, xe = 2 * x1 - 2;
+    if (xo < g.Un[n]) term(xo, d, A(1), TLevel<P, C>(pl, q, n).row(xo, kk));
+    if (2 * x1 < g.Un[n]) term(2 * x1, 0, A(0.5), nullptr);
+    if (x1 >= 2 && xe < g.Un[n]) term(xe, 2 * d, A(0.5), TLevel<P, C>(pl, q, n + 1).row(x1 - 1, 2 * kk));
+    A *o = gR1.base + gR1.idx(x1, j, 0, w);
+#pragma unroll
+    for (int c = 0; c < C; ++c) st4(o + c * Vs, acc[c]);
 }
 
 // ---------------------------------------------------------------------------
@@ -243,6 +361,58 @@ __device__ __forceinline__ void adj_T_part(const Plan &pl, int q, int n, int x, 
         GRLevel<P, C> gRm(pl, q, m);
         const bool rq = (n < g.N) && x + 1 < g.Un[n];
         RLevel<P, C> Rn(pl, q, rq ? n : 0);
+        if (k >= 2) cone(gRm, 2 * x, (k >> 1) - 1, A(0.5) * arc<P>(pl, n, k - 1), A(0.5), rq, Rn, x + 1, k - 1, n);
+        if (k < s) cone(gRm, 2 * x, k >> 1, A(0.5) * arc<P>(pl, n, k), A(0.5), rq, Rn, x + 1, k, n);
+    }
+}
+
+// adj_T_part for four consecutive v (n >= 1); entries past V are computed from
+// the padding and never read.
+template <int P, int C, bool ENV>
+__device__ __forceinline__ void adj_T_quad(const Plan &pl, int q, int n, int x, int k, int v,
+                                           typename Prec<P>::A (&gL)[C][4], typename Prec<P>::A (&gT)[4]) {
+    using A = typename Prec<P>::A;
+    const QuadGeom &g = pl.q[q];
+    const int s = 1 << n, d = 2 * k - s, V = g.V, Vs = g.Vs;
+#pragma unroll
+    for (int l = 0; l < 4; ++l) {
+        gT[l] = A(0);
+#pragma unroll
+        for (int c = 0; c < C; ++c) gL[c][l] = A(0);
+    }
+    auto cone = [&](const GRLevel<P, C> &gR, int xg, int ip, A Aw, A dw, bool rq, const RLevel<P, C> &R, int xr, int j,
+                    int rl) {
+        const A *gp = gR.base + gR.idx(xg, ip, 0, v);
+        const typename Prec<P>::SL *rp = R.base + R.idx(rq ? xr : 0, rq ? j : 0, 0, 0);
+        A dot[4] = {A(0), A(0), A(0), A(0)}, gr[C][4], r[C][4], ev[C];
+#pragma unroll
+        for (int c = 0; c < C; ++c) {
+            ev[c] = renv<P, C, ENV>(pl, q, rl, j, c);
+            ld4(gp + c * Vs, gr[c]);
+        }
+        rows4<C>(rq, rp, Vs, v + d, V, ev, r);
+#pragma unroll
+        for (int c = 0; c < C; ++c)
+#pragma unroll
+            for (int l = 0; l < 4; ++l) {
+                gL[c][l] = fma(Aw, gr[c][l], gL[c][l]);
+                dot[l] = fma(gr[c][l], r[c][l], dot[l]);
+            }
+#pragma unroll
+        for (int l = 0; l < 4; ++l) gT[l] = fma(dw, dot[l], gT[l]);
+    };
+    if ((x & 1) && n < g.N) {
+        const GRLevel<P, C> gRn(pl, q, n);
+        const int xq = (x + 1) >> 1;
+        const bool rq = (n + 1 < g.N) && xq < g.Un[n + 1];
+        const RLevel<P, C> R1(pl, q, rq ? n + 1 : n);
+        if (k >= 1) cone(gRn, x, k - 1, arc<P>(pl, n + 1, 2 * k - 1), A(1), rq, R1, xq, 2 * k - 1, n + 1);
+        if (k < s) cone(gRn, x, k, arc<P>(pl, n + 1, 2 * k), A(1), rq, R1, xq, 2 * k, n + 1);
+    }
+    if (!(k & 1)) {
+        const GRLevel<P, C> gRm(pl, q, n - 1);
+        const bool rq = (n < g.N) && x + 1 < g.Un[n];
+        const RLevel<P, C> Rn(pl, q, rq ? n : 0);
         if (k >= 2) cone(gRm, 2 * x, (k >> 1) - 1, A(0.5) * arc<P>(pl, n, k - 1), A(0.5), rq, Rn, x + 1, k - 1, n);
         if (k < s) cone(gRm, 2 * x, k >> 1, A(0.5) * arc<P>(pl, n, k), A(0.5), rq, Rn, x + 1, k, n);
     }
@@ -363,6 +533,93 @@ __device__ __forceinline__ void body_adj_merge_up(const Plan &pl, const RowSplit
         }
     }
     gTm.store2(x1, kap, w, aL, aT);           // w even, w + 1 < Vs
+}
+
+// body_adj_T (n >= 1) and body_adj_merge_up with four consecutive v per thread.
+template <int P, int C, bool ENV>
+__device__ __forceinline__ void body_adj_T4(const Plan &pl, const RowSplitB &rs, int n, long long bx, int by) {
+    using A = typename Prec<P>::A;
+    int local;
+    const int q = quadrant_of(rs, bx, local);
+    const QuadGeom &g = pl.q[q];
+    const int v = 4 * (by * blockDim.x + threadIdx.x);
+    if (v >= g.V) return;
+    const int K = (1 << n) + 1;
+    local += K;
+    const int x = local / K, k = local - x * K;
+    A gL[C][4], gT[4];
+    adj_T_quad<P, C, ENV>(pl, q, n, x, k, v, gL, gT);
+    A *o = GTLevel<P, C>(pl, q, n).row(x, k) + v;
+#pragma unroll
+    for (int c = 0; c < C; ++c) st4(o + c * g.Vs, gL[c]);
+    st4(o + C * g.Vs, gT);
+}
+
+template <int P, int C, bool ENV>
+__device__ __forceinline__ void body_adj_merge_up4(const Plan &pl, const RowSplitB &rs, int n, long long bx, int by) {
+    using A = typename Prec<P>::A;
+    int local;
+    const int q = quadrant_of(rs, bx, local);   // row = (q, x', kap) at level n-1
+    const QuadGeom &g = pl.q[q];
+    const int w = 4 * (by * blockDim.x + threadIdx.x), V = g.V, Vs = g.Vs;
+    if (w >= V) return;
+    const int m = n - 1, h = 1 << m;
+    local += h + 1;                               // x' >= 1: column 0 is dead
+    const int x1 = local / (h + 1), kap = local - x1 * (h + 1);
+    const TLevel<P, C> Tm(pl, q, m);
+    const GTLevel<P, C> gTm(pl, q, m), gTn(pl, q, n);
+    A aL[C][4], aT[4];
+    adj_T_quad<P, C, ENV>(pl, q, m, x1, kap, w, aL, aT);
+    if (!(x1 & 1)) {
+        const int x = x1 >> 1, xf = x1 + 1, vf = w + 2 * kap - h;
+        const bool xok = xf < g.Un[m];
+#pragma unroll
+        for (int t = 0; t < 3; ++t) {
+            const int kout = t == 0 ? 2 * kap : (t == 1 ? 2 * kap + 1 : 2 * kap - 1);
+            const int fdir = t == 0 ? kap : (t == 1 ? kap + 1 : kap - 1);
+            if (kout < 0 || kout > 2 * h) continue;
+            const A wgt = t == 0 ? A(1) : A(0.5);
+            const A *gr = gTn.row(x, kout) + w;
+            A dT[4], f[C][4], gv[C + 1][4];
+#pragma unroll
+            for (int c = 0; c <= C; ++c) ld4(gr + c * Vs, gv[c]);
+            interval4<P, C>(xok, Tm.row(xok ? xf : x1, fdir), Vs, vf, V, f, dT);
+#pragma unroll
+            for (int l = 0; l < 4; ++l) dT[l] = gv[C][l] * dT[l];
+#pragma unroll
+            for (int c = 0; c < C; ++c)
+#pragma unroll
+                for (int l = 0; l < 4; ++l) {
+                    aL[c][l] = fma(wgt, gv[c][l], aL[c][l]);
+                    dT[l] = fma(gv[c][l], f[c][l], dT[l]);
+                }
+#pragma unroll
+            for (int l = 0; l < 4; ++l) aT[l] = fma(wgt, dT[l], aT[l]);
+        }
+    } else if (x1 >= 3) {                         // x' = 1 is the far operand of the dead column 0
+        const int x = (x1 - 1) >> 1, xn = x1 - 1;
+#pragma unroll
+        for (int t = 0; t < 3; ++t) {
+            const int kout = t == 0 ? 2 * kap : (t == 1 ? 2 * kap + 1 : 2 * kap - 1);
+            const int ndir = t == 0 ? kap : (t == 1 ? kap + 1 : kap - 1);
+            if (kout < 0 || kout > 2 * h) continue;
+            const int v = w - (2 * ndir - h);
+            const A wgt = t == 0 ? A(1) : A(0.5);
+            A tn[4], gv[C + 1][4];
+            shifted4<P, C, C + 1>(true, Tm.row(xn, ndir), gTn.row(x, kout), Vs, v, V, tn, gv);
+#pragma unroll
+            for (int l = 0; l < 4; ++l) {
+                tn[l] = wgt * tn[l];
+#pragma unroll
+                for (int c = 0; c < C; ++c) aL[c][l] = fma(tn[l], gv[c][l], aL[c][l]);
+                aT[l] = fma(tn[l], gv[C][l], aT[l]);
+            }
+        }
+    }
+    A *o = gTm.row(x1, kap) + w;
+#pragma unroll
+    for (int c = 0; c < C; ++c) st4(o + c * Vs, aL[c]);
+    st4(o + C * Vs, aT);
 }
 
 // ---------------------------------------------------------------------------

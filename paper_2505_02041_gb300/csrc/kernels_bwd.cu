@@ -21,28 +21,53 @@ __device__ __forceinline__ void row_block_b(const Plan &pl, long long &row, int 
     else { row = blockIdx.x; vb = blockIdx.y; }
 }
 
-template <int P, int C, int E>
-__global__ void __launch_bounds__(512) k_adj_R(Plan pl, RowSplitB rs, int n) {
+// Level 0 (odd shifts): one v per thread.
+template <int P, int C>
+__global__ void __launch_bounds__(512) k_adj_R0(Plan pl, RowSplitB rs, int n) {
     long long row;
     int vb;
     row_block_b(pl, row, vb);
-    body_adj_R<P, C, E>(pl, rs, n, row, vb);
-}
-
-template <int P, int C, int E, bool ENV>
-__global__ void __launch_bounds__(512) k_adj_T(Plan pl, RowSplitB rs, int n) {
-    long long row;
-    int vb;
-    row_block_b(pl, row, vb);
-    body_adj_T<P, C, E, ENV>(pl, rs, n, row, vb);
+    body_adj_R<P, C, 1>(pl, rs, n, row, vb);
 }
 
 template <int P, int C, bool ENV>
-__global__ void __launch_bounds__(512) k_adj_merge_up(Plan pl, RowSplitB rs, int n) {
+__global__ void __launch_bounds__(512) k_adj_T0(Plan pl, RowSplitB rs, int n) {
     long long row;
     int vb;
     row_block_b(pl, row, vb);
-    body_adj_merge_up<P, C, ENV>(pl, rs, n, row, vb);
+    body_adj_T<P, C, 1, ENV>(pl, rs, n, row, vb);
+}
+
+// Levels n >= 1: four v per thread.  These kernels issue in about 65 % of the
+// slots, most of it addresses and range tests, so a thread that shares them
+// over four entries is faster than one of two -- provided that a shifted
+// range is tested once for all its rows (rows4, shifted4, interval4): with a
+// test per channel the merge-up reverse took 513 us instead of 387 (1024^2,
+// C = 3, fp32).  Pairs -> quads, us, C = 3 / C = 1 at 1024^2 fp32: merge-down
+// reverse 272 -> 247 / 188 -> 144, merge-up reverse 374 -> 366 / 260 -> 196;
+// bf16 C = 3: 277 -> 240, 354 -> 323.
+template <int P, int C>
+__global__ void __launch_bounds__(512) k_adj_R4(Plan pl, RowSplitB rs, int n) {
+    long long row;
+    int vb;
+    row_block_b(pl, row, vb);
+    body_adj_R4<P, C>(pl, rs, n, row, vb);
+}
+
+template <int P, int C, bool ENV>
+__global__ void __launch_bounds__(512) k_adj_T4(Plan pl, RowSplitB rs, int n) {
+    long long row;
+    int vb;
+    row_block_b(pl, row, vb);
+    body_adj_T4<P, C, ENV>(pl, rs, n, row, vb);
+}
+
+template <int P, int C, bool ENV>
+__global__ void __launch_bounds__(512) k_adj_merge_up4(Plan pl, RowSplitB rs, int n) {
+    long long row;
+    int vb;
+    row_block_b(pl, row, vb);
+    body_adj_merge_up4<P, C, ENV>(pl, rs, n, row, vb);
 }
 
 template <int P, int C, class IN>
@@ -189,8 +214,8 @@ static cudaError_t bwd_impl(const Plan &pl, const RayTable &rt, const void *e, c
                 by += gRbytes(q, n) + gRbytes(q, n + 1) + bytes_T(pl, q, n) / (pl.C + 1) / 2 +
                       bytes_T(pl, q, n + 1) / (pl.C + 1) / 2;
         rec->begin(K_ADJ_MERGE_DOWN, n, by);
-        if (n >= 1) k_adj_R<P, C, 2><<<row_grid_b(pl, rs.start[4], 2 * mt), mt, 0, st>>>(pl, rs, n);
-        else k_adj_R<P, C, 1><<<row_grid_b(pl, rs.start[4], ts), ts, 0, st>>>(pl, rs, n);
+        if (n >= 1) k_adj_R4<P, C><<<row_grid_b(pl, rs.start[4], 4 * mt), mt, 0, st>>>(pl, rs, n);
+        else k_adj_R0<P, C><<<row_grid_b(pl, rs.start[4], ts), ts, 0, st>>>(pl, rs, n);
         rec->end();
         ++*launches;
     }
@@ -203,11 +228,11 @@ static cudaError_t bwd_impl(const Plan &pl, const RayTable &rt, const void *e, c
                 by += gTbytes(q, n) + gRbytes(q, n) + gRbytes(q, n - 1) + bytes_R(pl, q, n) + bytes_R(pl, q, n + 1);
         rec->begin(K_ADJ_MERGE_DOWN, n, by);
         if (n >= 1) {
-            if (env) k_adj_T<P, C, 2, true><<<row_grid_b(pl, rs.start[4], 2 * mt), mt, 0, st>>>(pl, rs, n);
-            else k_adj_T<P, C, 2, false><<<row_grid_b(pl, rs.start[4], 2 * mt), mt, 0, st>>>(pl, rs, n);
+            if (env) k_adj_T4<P, C, true><<<row_grid_b(pl, rs.start[4], 4 * mt), mt, 0, st>>>(pl, rs, n);
+            else k_adj_T4<P, C, false><<<row_grid_b(pl, rs.start[4], 4 * mt), mt, 0, st>>>(pl, rs, n);
         } else {
-            if (env) k_adj_T<P, C, 1, true><<<row_grid_b(pl, rs.start[4], ts), ts, 0, st>>>(pl, rs, n);
-            else k_adj_T<P, C, 1, false><<<row_grid_b(pl, rs.start[4], ts), ts, 0, st>>>(pl, rs, n);
+            if (env) k_adj_T0<P, C, true><<<row_grid_b(pl, rs.start[4], ts), ts, 0, st>>>(pl, rs, n);
+            else k_adj_T0<P, C, false><<<row_grid_b(pl, rs.start[4], ts), ts, 0, st>>>(pl, rs, n);
         }
         rec->end();
         ++*launches;
@@ -221,8 +246,8 @@ static cudaError_t bwd_impl(const Plan &pl, const RayTable &rt, const void *e, c
                 by += gTbytes(q, n - 1) + gTbytes(q, n) + bytes_T(pl, q, n - 1) + gRbytes(q, n - 1) +
                       gRbytes(q, n - 2) + bytes_R(pl, q, n - 1) + bytes_R(pl, q, n);
         rec->begin(K_ADJ_MERGE_UP, n, by);
-        if (env) k_adj_merge_up<P, C, true><<<row_grid_b(pl, rs.start[4], 2 * mt), mt, 0, st>>>(pl, rs, n);
-        else k_adj_merge_up<P, C, false><<<row_grid_b(pl, rs.start[4], 2 * mt), mt, 0, st>>>(pl, rs, n);
+        if (env) k_adj_merge_up4<P, C, true><<<row_grid_b(pl, rs.start[4], 4 * mt), mt, 0, st>>>(pl, rs, n);
+        else k_adj_merge_up4<P, C, false><<<row_grid_b(pl, rs.start[4], 4 * mt), mt, 0, st>>>(pl, rs, n);
         rec->end();
         ++*launches;
     }

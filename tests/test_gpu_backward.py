@@ -209,3 +209,29 @@ def test_adjoint_trace_forms(W, H, C, casc, seed):
         ge_r, gs_r = oracle.fluence_adjoint(e, s, gF, casc)
         ge, gs = _gpu_grads(e.astype(np.float64), s.astype(np.float64), gF, "fp64", casc)
         assert err_max(ge, ge_r) <= 1e-10 and err_max(gs, gs_r) <= 1e-10
+
+
+@pytest.mark.parametrize("W,H,C,prec", [
+    (62, 61, 3, "fp32"), (131, 70, 1, "fp32"), (33, 258, 4, "fp32"), (4, 9, 2, "fp32"), (129, 66, 3, "bf16"), (60, 47, 1, "fp16"),
+])
+def test_adjoint_quads_match_pairs(W, H, C, prec):
+    """The single-scene adjoint kernels take four v per thread, the batched
+    persistent launch two: rows of every length mod 4 (quads straddling the end
+    of a row, shifts that are and are not multiples of 4).  Each entry's
+    arithmetic is the same; only the order of the last sum over the frames
+    may differ, a few fp32 roundings (2^-24 each) of the largest value."""
+    require_gpu()
+    from paper_2505_02041_gb300 import HRC, BatchedHRC
+    e, s = scenes.random_scene(W, H, C, 97)
+    gF = scenes.rng(98).normal(size=e.shape).astype(np.float32)
+    ed, sd, gd = to_dev(e), to_dev(s), to_dev(gF)
+    h = HRC(W, H, C, 0, prec)
+    h.forward(ed, sd)
+    ge, gs = h.backward(gd)
+    b = BatchedHRC([(W, H)], C, 0, prec)
+    b.tune(0, 0, 0)
+    b.forward(ed.reshape(-1), sd.reshape(-1))
+    geb, gsb = b.backward(gd.reshape(-1))
+    b.sync()
+    assert err_max(ge.cpu().numpy().reshape(-1), geb.cpu().numpy()) <= 1e-6
+    assert err_max(gs.cpu().numpy().reshape(-1), gsb.cpu().numpy()) <= 1e-6
