@@ -134,7 +134,10 @@ hrc_status hrc_set_schedule(hrc_ctx *ctx, int schedule);
  *             level-to-level dependencies are tracked by per-column
  *             completion counters with bounded waits; not with schedule 2).
  *             FP64 always uses 0.
- * Defaults {0, 1, 128, 0, 0}; hrc_autotune picks one. */
+ * Defaults {0, 1, 128, 0, 0}; hrc_autotune picks one.  Until a configuration
+ * is set or autotuned, a context of 384^2 pixels and more runs its merge
+ * kernels with groups 4 and grid order 1 (where that is allowed); the values
+ * read back are the defaults all the same. */
 typedef struct hrc_launch_config {
     int schedule, groups, threads, vmajor, mdown;
 } hrc_launch_config;

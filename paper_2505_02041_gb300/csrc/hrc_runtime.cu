@@ -182,6 +182,7 @@ struct hrc_ctx {
     int mthreads = 128;
     int vmajor = 0;
     int mdown = 0;
+    bool cfg_set = false;        // a launch configuration was set or autotuned (else own_config decides)
     int device = 0;
     cudaStream_t stream = nullptr;
     RayTable rt;
@@ -344,6 +345,23 @@ cudaError_t upload_arcs(const Plan &pl, char *arena) {
     return cudaMemcpy(arena + pl.arcs_off_d, ad.data(), ad.size() * sizeof(double), cudaMemcpyHostToDevice);
 }
 
+// The plan of a pass in a context whose launch configuration nobody has set:
+// on grids of 384^2 pixels and more the merge up takes four v per thread and
+// the v-blocks of a row are adjacent in launch order, the autotuner's choice at
+// nearly every such size (forward in fp32, C = 3, us, the initial
+// configuration / this one: 512^2 113.0 / 110.9, 768^2 257.5 / 253.8, 1024^2
+// 484 / 461, 2048^2 2028 / 1888; bf16 2048^2 2046 / 1737).  Below, half the threads
+// cost more than the wider loads save (256^2: 49.2 / 49.3, C = 1 41.0 / 41.7).
+Plan own_config(const hrc_ctx *ctx, const Plan &base) {
+    Plan pl = base;
+    if (!ctx->cfg_set && (long long)ctx->W * ctx->H >= 384LL * 384 && ctx->prec != P_FP64) {
+        pl.mgroups = 4;
+        if (4LL * (ctx->W + ctx->H) <= 65535) pl.vmajor = 1;
+    }
+    return pl;
+}
+int groups_key(const hrc_ctx *ctx) { return ctx->mgroups + (ctx->cfg_set ? 16 : 0); }
+
 // Enqueue one pass (forward or backward) on the context's stream: replay its
 // CUDA graph when one exists for these pointers, capture one otherwise.
 // With per-launch timing on, the kernels are launched directly.
@@ -371,7 +389,7 @@ hrc_status run_pass_key(hrc_ctx *ctx, int kind, const PassKey &pk, ENQ &&enqueue
     const bool timed = ctx->rec.on;
     const void *const *key = pk.p;
     for (auto &g : ctx->graphs) {
-        if (g.exec && g.kind == kind && g.prec == ctx->prec && g.sched == ctx->sched && g.mgroups == ctx->mgroups &&
+        if (g.exec && g.kind == kind && g.prec == ctx->prec && g.sched == ctx->sched && g.mgroups == groups_key(ctx) &&
             g.tune == ctx->mthreads * 8 + ctx->vmajor * 4 + ctx->mdown && g.timed == (timed ? ctx->timing_mode : 0) &&
             std::memcmp(g.p, key, sizeof(pk.p)) == 0) {
             cudaError_t e = cudaGraphLaunch(g.exec, ctx->stream);
@@ -394,7 +412,7 @@ hrc_status run_pass_key(hrc_ctx *ctx, int kind, const PassKey &pk, ENQ &&enqueue
         mix((unsigned long long)kind);
         mix((unsigned long long)ctx->prec);
         mix((unsigned long long)ctx->sched);
-        mix((unsigned long long)ctx->mgroups);
+        mix((unsigned long long)groups_key(ctx));
         mix((unsigned long long)(ctx->mthreads * 8 + ctx->vmajor * 4 + ctx->mdown));
         for (int i = 0; i < 8; ++i) mix((unsigned long long)(uintptr_t)key[i]);
         int unreplayed = 0;
@@ -447,7 +465,7 @@ hrc_status run_pass_key(hrc_ctx *ctx, int kind, const PassKey &pk, ENQ &&enqueue
     slot.kind = kind;
     slot.prec = ctx->prec;
     slot.sched = ctx->sched;
-    slot.mgroups = ctx->mgroups;
+    slot.mgroups = groups_key(ctx);
     slot.tune = ctx->mthreads * 8 + ctx->vmajor * 4 + ctx->mdown;
     slot.timed = timed ? ctx->timing_mode : 0;
     slot.recs = timed ? ctx->rec.recs : std::vector<Recorder::Rec>();
@@ -814,6 +832,7 @@ hrc_status hrc_set_launch_config(hrc_ctx *ctx, const hrc_launch_config *cfg) {
     if (ctx->batched) return fail(ctx, HRC_EINVAL, "hrc_set_launch_config: single-scene contexts only");
     if (!config_valid(ctx, *cfg)) return fail(ctx, HRC_EINVAL, "hrc_set_launch_config: value out of range");
     apply_config(ctx, *cfg);
+    ctx->cfg_set = true;
     ctx->have_fwd = false;
     for (hrc_ctx *k : ctx->chan) hrc_set_launch_config(k, cfg);
     return HRC_OK;
@@ -843,6 +862,7 @@ hrc_status hrc_autotune(hrc_ctx *ctx, float *best_ms) {
     hrc_get_launch_config(ctx, &best_c);
     const bool timing = ctx->rec.on;
     ctx->rec.on = false;
+    ctx->cfg_set = true;
     static const int kThreads[4] = {64, 128, 256, 512};
     static const int kGroups[3] = {1, 2, 4};
     for (int cand = 0; cand < 3 * 3 * 4 * 2 * 3 && st == HRC_OK; ++cand) {
@@ -1108,6 +1128,7 @@ hrc_status hrc_set_channel_extinction(hrc_ctx *ctx, int per_channel) {
             if (st == HRC_OK) st = hrc_set_stream(k, ctx->stream);
             if (st == HRC_OK) st = hrc_set_precision(k, (hrc_precision)ctx->prec);
             if (st == HRC_OK) st = hrc_set_launch_config(k, &cfg);
+            if (st == HRC_OK) k->cfg_set = ctx->cfg_set;
             if (st == HRC_OK) st = hrc_set_backward_recompute(k, ctx->bwd_recompute ? 1 : 0);
             if (st == HRC_OK && ctx->blur_buf) st = hrc_set_cross_blur(k, ctx->blur ? 1 : 0, ctx->blur_thr);
             if (st == HRC_OK && ctx->bounce_buf) st = hrc_reserve_bounces(k, ctx->bounce_cap);
@@ -1237,7 +1258,7 @@ hrc_status hrc_fluence(hrc_ctx *ctx, const float *emission, const float *sigma_t
     if (!emission || !sigma_t || !out) return fail(ctx, HRC_EINVAL, "hrc_fluence: NULL pointer");
     if (!aligned16(emission) || !aligned16(sigma_t) || !aligned16(out))
         return fail(ctx, HRC_EINVAL, "hrc_fluence: pointers must be 16-byte aligned");
-    const Plan pl = ctx->plan;
+    const Plan pl = own_config(ctx, ctx->plan);
     const RayTable *rt = &ctx->rt;
     void *Fr = ctx->blur ? ctx->blur_buf : nullptr;
     const double thr = ctx->blur_thr;
@@ -1317,7 +1338,7 @@ hrc_status hrc_fluence_backward(hrc_ctx *ctx, const float *grad_F, float *grad_e
     if (!grad_F || !grad_emission || !grad_sigma_t) return fail(ctx, HRC_EINVAL, "hrc_fluence_backward: NULL pointer");
     if (!aligned16(grad_F) || !aligned16(grad_emission) || !aligned16(grad_sigma_t))
         return fail(ctx, HRC_EINVAL, "hrc_fluence_backward: pointers must be 16-byte aligned");
-    const Plan pl = ctx->plan;
+    const Plan pl = own_config(ctx, ctx->plan);
     const RayTable *rt = &ctx->rt;
     const void *le = ctx->last_e, *ls = ctx->last_s;
     const bool rc = ctx->bwd_recompute;
@@ -1414,7 +1435,7 @@ hrc_status bounces_forward(hrc_ctx *ctx, const void *e, const void *s, const voi
     if (!ctx->bounce_buf) return fail(ctx, HRC_ESTATE, std::string(where) + ": call hrc_reserve_bounces first");
     if (K < 0 || K > ctx->bounce_cap)
         return fail(ctx, HRC_EINVAL, std::string(where) + ": bounces must be in [0, the count reserved by hrc_reserve_bounces]");
-    const Plan pl = f64 ? ctx->plan64 : ctx->plan;
+    const Plan pl = f64 ? ctx->plan64 : own_config(ctx, ctx->plan);
     const RayTable *rt = &ctx->rt;
     void *blur = ctx->blur ? ctx->blur_buf : nullptr;
     const double thr = ctx->blur_thr;
@@ -1453,7 +1474,7 @@ hrc_status bounces_backward(hrc_ctx *ctx, const void *gF, void *ge, void *gs, vo
     if (!gF || !ge || !gs || !ga) return fail(ctx, HRC_EINVAL, std::string(where) + ": NULL pointer");
     if (!aligned16(gF) || !aligned16(ge) || !aligned16(gs) || !aligned16(ga))
         return fail(ctx, HRC_EINVAL, std::string(where) + ": pointers must be 16-byte aligned");
-    const Plan pl = f64 ? ctx->plan64 : ctx->plan;
+    const Plan pl = f64 ? ctx->plan64 : own_config(ctx, ctx->plan);
     const RayTable *rt = &ctx->rt;
     void *blur = ctx->blur ? ctx->blur_buf : nullptr;
     const double thr = ctx->blur_thr;
