@@ -418,6 +418,136 @@ __device__ __forceinline__ void adj_T_quad(const Plan &pl, int q, int n, int x, 
     }
 }
 
+// Level 0 with four consecutive v per thread.  Its shifts are +-1 (T_0 and
+// R_1 against odd columns) and +-2 (even columns): a run of four starting
+// there is the aligned four at w and the one or two entries beyond it.
+
+// r[c] = plane c at w + o .. w + o + 3, o = -2, -1, 1 or 2 (zero shifts need no
+// helper), entries outside [0, V) ev[c]; planes `stride` apart, w a multiple of
+// 4 and w < V.
+template <int NC, class S, class A>
+__device__ __forceinline__ void beside4(bool ok, const S *row, int stride, int w, int o, int V, const A (&ev)[NC],
+                                        A (&r)[NC][4]) {
+    A b[NC][2];
+#pragma unroll
+    for (int c = 0; c < NC; ++c) {
+        b[c][0] = b[c][1] = ev[c];
+#pragma unroll
+        for (int l = 0; l < 4; ++l) r[c][l] = ev[c];
+    }
+    if (ok) {
+#pragma unroll
+        for (int c = 0; c < NC; ++c) ld4(row + (long long)c * stride + w, r[c]);
+        if (o > 0 ? w + 4 < V : w >= 4) {
+            const int p = o > 0 ? w + 4 : w - 2;
+#pragma unroll
+            for (int c = 0; c < NC; ++c) ld2(row + (long long)c * stride + p, b[c][0], b[c][1]);
+        }
+        if (w + 5 >= V) {                       // the row ends inside the run
+#pragma unroll
+            for (int c = 0; c < NC; ++c) {
+                if (o > 0) b[c][1] = ev[c];
+#pragma unroll
+                for (int l = 1; l < 4; ++l)
+                    if (w + l >= V) r[c][l] = ev[c];
+            }
+        }
+    }
+#pragma unroll
+    for (int c = 0; c < NC; ++c) {
+        const A x[8] = {b[c][0], b[c][1], r[c][0], r[c][1], r[c][2], r[c][3], b[c][0], b[c][1]};
+#pragma unroll
+        for (int l = 0; l < 4; ++l)
+            r[c][l] = o == -2 ? x[l] : (o == -1 ? x[l + 1] : (o == 1 ? x[l + 3] : x[l + 4]));
+    }
+}
+
+// dL/dR_1(x', j, w .. w + 3) from dL/dR_0 (body_adj_R at n = 0).
+template <int P, int C>
+__device__ __forceinline__ void body_adj_R0(const Plan &pl, const RowSplitB &rs, long long bx, int by) {
+    using A = typename Prec<P>::A;
+    using SL = typename Prec<P>::SL;
+    using ST = typename Prec<P>::ST;
+    int local;
+    const int q = quadrant_of(rs, bx, local);
+    const QuadGeom &g = pl.q[q];
+    const int w = 4 * (by * blockDim.x + threadIdx.x), V = g.V, Vs = g.Vs;
+    if (w >= V) return;
+    local += 2;
+    const int x1 = local >> 1, j = local & 1, d = 2 * j - 1;   // ip = 0, kk = j
+    const GRLevel<P, C> gR0(pl, q, 0), gR1(pl, q, 1);
+    const A zero[C] = {}, vac[1] = {Prec<P>::LOG ? A(0) : A(1)};
+    A acc[C][4];
+#pragma unroll
+    for (int c = 0; c < C; ++c)
+#pragma unroll
+        for (int l = 0; l < 4; ++l) acc[c][l] = A(0);
+    // + weight T(xt, kt) gR_0(xp, 0) at w - sh
+    auto term = [&](int xp, int sh, A wgt, const char *trow) {
+        A t[1][4], r[C][4];
+        beside4<C>(true, gR0.base + gR0.idx(xp, 0, 0, 0), Vs, w, -sh, V, zero, r);
+        beside4<1>(true, reinterpret_cast<const ST *>(trow + (size_t)C * Vs * sizeof(SL)), Vs, w, -sh, V, vac, t);
+#pragma unroll
+        for (int l = 0; l < 4; ++l) {
+            const A tw = wgt * (Prec<P>::LOG ? fexp(-t[0][l]) : t[0][l]);
+#pragma unroll
+            for (int c = 0; c < C; ++c) acc[c][l] = fma(tw, r[c][l], acc[c][l]);
+        }
+    };
+    const int xo = 2 * x1 - 1, xe = 2 * x1 - 2;
+    if (xo < g.U) term(xo, d, A(1), TLevel<P, C>(pl, q, 0).row(xo, j));
+    if (2 * x1 < g.U) {
+        const A *gp = gR0.base + gR0.idx(2 * x1, 0, 0, w);
+#pragma unroll
+        for (int c = 0; c < C; ++c) {
+            A r[4];
+            ld4(gp + c * Vs, r);
+#pragma unroll
+            for (int l = 0; l < 4; ++l) acc[c][l] = fma(A(0.5), r[l], acc[c][l]);
+        }
+    }
+    if (x1 >= 2 && xe < g.U) term(xe, 2 * d, A(0.5), TLevel<P, C>(pl, q, 1).row(x1 - 1, 2 * j));
+    A *o = gR1.base + gR1.idx(x1, j, 0, w);
+#pragma unroll
+    for (int c = 0; c < C; ++c) st4(o + c * Vs, acc[c]);
+}
+
+// dL/dT_0(x, k, v .. v + 3) at odd x (body_adj_T at n = 0): the cone of level 0
+// with R_1((x + 1) / 2, k) at v + 2 k - 1.
+template <int P, int C, bool ENV>
+__device__ __forceinline__ void body_adj_T0(const Plan &pl, const RowSplitB &rs, long long bx, int by) {
+    using A = typename Prec<P>::A;
+    int local;
+    const int q = quadrant_of(rs, bx, local);
+    const QuadGeom &g = pl.q[q];
+    const int v = 4 * (by * blockDim.x + threadIdx.x), Vs = g.Vs;
+    if (v >= g.V) return;
+    const int x = 2 * (local >> 1) + 1, k = local & 1, xq = (x + 1) >> 1;
+    const bool rq = 1 < g.N && xq < g.Un[1];
+    const GRLevel<P, C> gR0(pl, q, 0);
+    const RLevel<P, C> R1(pl, q, rq ? 1 : 0);
+    const A Aw = arc<P>(pl, 1, k);
+    A gr[C][4], r[C][4], ev[C], gT[4] = {A(0), A(0), A(0), A(0)};
+#pragma unroll
+    for (int c = 0; c < C; ++c) {
+        ev[c] = renv<P, C, ENV>(pl, q, 1, k, c);
+        ld4(gR0.base + gR0.idx(x, 0, c, v), gr[c]);
+    }
+    beside4<C>(rq, R1.base + R1.idx(rq ? xq : 0, rq ? k : 0, 0, 0), Vs, v, 2 * k - 1, g.V, ev, r);
+    A *o = GTLevel<P, C>(pl, q, 0).row(x, k) + v;
+#pragma unroll
+    for (int c = 0; c < C; ++c) {
+        A gl[4];
+#pragma unroll
+        for (int l = 0; l < 4; ++l) {
+            gT[l] = fma(gr[c][l], r[c][l], gT[l]);
+            gl[l] = fma(Aw, gr[c][l], A(0));
+        }
+        st4(o + c * Vs, gl);
+    }
+    st4(o + C * Vs, gT);
+}
+
 // Levels whose merge-down part is computed inside the merge-up reverse of
 // the level above (n = 2 .. N-1); adj_T covers the others.
 __host__ __device__ inline bool adj_T_fused(int n, int N) { return n >= 2 && n <= N - 1; }

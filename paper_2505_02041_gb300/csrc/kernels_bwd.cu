@@ -21,21 +21,21 @@ __device__ __forceinline__ void row_block_b(const Plan &pl, long long &row, int 
     else { row = blockIdx.x; vb = blockIdx.y; }
 }
 
-// Level 0 (odd shifts): one v per thread.
+// Level 0 (odd shifts), four v per thread like the levels above.
 template <int P, int C>
-__global__ void __launch_bounds__(512) k_adj_R0(Plan pl, RowSplitB rs, int n) {
+__global__ void __launch_bounds__(512) k_adj_R0(Plan pl, RowSplitB rs) {
     long long row;
     int vb;
     row_block_b(pl, row, vb);
-    body_adj_R<P, C, 1>(pl, rs, n, row, vb);
+    body_adj_R0<P, C>(pl, rs, row, vb);
 }
 
 template <int P, int C, bool ENV>
-__global__ void __launch_bounds__(512) k_adj_T0(Plan pl, RowSplitB rs, int n) {
+__global__ void __launch_bounds__(512) k_adj_T0(Plan pl, RowSplitB rs) {
     long long row;
     int vb;
     row_block_b(pl, row, vb);
-    body_adj_T<P, C, 1, ENV>(pl, rs, n, row, vb);
+    body_adj_T0<P, C, ENV>(pl, rs, row, vb);
 }
 
 // Levels n >= 1: four v per thread.  These kernels issue in about 65 % of the
@@ -172,7 +172,7 @@ template <int P, int C>
 static cudaError_t bwd_impl(const Plan &pl, const RayTable &rt, const void *e, const void *s, const void *gF,
                             void *ge, void *gs, bool recompute, cudaStream_t st, int *launches, Recorder *rec) {
     using IN = typename std::conditional<P == P_FP64, double, float>::type;
-    const int mt = pl.mthreads, ts = 2 * mt > 512 ? 512 : 2 * mt;   // paired-v / single-v block sizes
+    const int mt = pl.mthreads;
     const bool env = plan_has_env(pl);   // kernels compiled for an environment map
     int Nmax = 0, Nmin = pl.q[0].N;
     for (int q = 0; q < 4; ++q) {
@@ -215,7 +215,7 @@ static cudaError_t bwd_impl(const Plan &pl, const RayTable &rt, const void *e, c
                       bytes_T(pl, q, n + 1) / (pl.C + 1) / 2;
         rec->begin(K_ADJ_MERGE_DOWN, n, by);
         if (n >= 1) k_adj_R4<P, C><<<row_grid_b(pl, rs.start[4], 4 * mt), mt, 0, st>>>(pl, rs, n);
-        else k_adj_R0<P, C><<<row_grid_b(pl, rs.start[4], ts), ts, 0, st>>>(pl, rs, n);
+        else k_adj_R0<P, C><<<row_grid_b(pl, rs.start[4], 4 * mt), mt, 0, st>>>(pl, rs);
         rec->end();
         ++*launches;
     }
@@ -231,8 +231,8 @@ static cudaError_t bwd_impl(const Plan &pl, const RayTable &rt, const void *e, c
             if (env) k_adj_T4<P, C, true><<<row_grid_b(pl, rs.start[4], 4 * mt), mt, 0, st>>>(pl, rs, n);
             else k_adj_T4<P, C, false><<<row_grid_b(pl, rs.start[4], 4 * mt), mt, 0, st>>>(pl, rs, n);
         } else {
-            if (env) k_adj_T0<P, C, true><<<row_grid_b(pl, rs.start[4], ts), ts, 0, st>>>(pl, rs, n);
-            else k_adj_T0<P, C, false><<<row_grid_b(pl, rs.start[4], ts), ts, 0, st>>>(pl, rs, n);
+            if (env) k_adj_T0<P, C, true><<<row_grid_b(pl, rs.start[4], 4 * mt), mt, 0, st>>>(pl, rs);
+            else k_adj_T0<P, C, false><<<row_grid_b(pl, rs.start[4], 4 * mt), mt, 0, st>>>(pl, rs);
         }
         rec->end();
         ++*launches;
