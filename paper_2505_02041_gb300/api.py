@@ -19,6 +19,10 @@ _PREC = {
 
 
 def _dev_tensor(t, dtype, shape, name):
+    # the usual case in one expression: these calls are made several times a
+    # pass, and a 256^2 gradient step takes longer on the host than on the GPU
+    if type(t) is torch.Tensor and t.is_cuda and t.dtype is dtype and t.shape == shape and t.is_contiguous():
+        return t if not t.data_ptr() & 15 else t.clone()
     if not isinstance(t, torch.Tensor) or not t.is_cuda:
         raise TypeError(f"{name} must be a CUDA tensor")
     if t.dtype != dtype:
@@ -62,7 +66,7 @@ class HRC:
         return torch.float64 if self.precision == "fp64" else torch.float32
 
     def _stream(self):
-        _lib.hrc_set_stream(self.ctx, torch.cuda.current_stream(self.device).cuda_stream)
+        _lib.hrc_set_stream(self.ctx, torch._C._cuda_getCurrentRawStream(self.device.index))
 
     # -- compute -----------------------------------------------------------
     def forward(self, emission, sigma_t, out=None):
