@@ -427,7 +427,7 @@ hrc_status hrc_batched_tune(hrc_ctx *ctx, int blocks_per_sm, int order);
  * one persistent launch that runs every scene's merge cascade from a
  * ticket queue with bounded dependency waits; 1 = every scene's own
  * per-level launch sequence (as a single-scene pass), the scenes spread
- * largest first over 8 streams forked from and joined to the caller's
+ * largest first over 8 or 16 streams forked from and joined to the caller's
  * stream, so that kernels of different scenes overlap; 2 = level-major
  * multi-scene launches: one launch per stage (each merge-up level, each
  * merge-down level, the fluence sum; each adjoint level) covering every

@@ -297,9 +297,9 @@ struct hrc_ctx {
     int blocks_per_sm = 0;              // 0: as many as fit
     int order = 0;                      // 0: scenes in input order per stage, 1: largest first
     // schedule 1: one graph whose branches are the scenes' per-level launch
-    // chains, spread over kAux streams (forked from and joined to the pass)
+    // chains, spread over up to kAux streams (forked from and joined to the pass)
     int bsched = 0;
-    static constexpr int kAux = 8;
+    static constexpr int kAux = 16;
     cudaStream_t aux[kAux] = {};
     cudaEvent_t ev_fork = nullptr, ev_join[kAux] = {};
     std::vector<int> by_size;           // scene indices, largest first
@@ -1739,14 +1739,22 @@ hrc_status build_batched_plans(hrc_ctx *ctx, int prec) {
 // independent branch per stream, so kernels of different scenes overlap.
 hrc_status run_batched_chains(hrc_ctx *ctx, int mode, const void *e, const void *s, void *F, const void *gF,
                               void *ge, void *gs, const char *where) {
+    // Branches: a small scene's kernels leave most of the GPU idle and follow
+    // each other at their own latency, so more chains at once help (96 scenes
+    // of 64^2-256^2, bf16, forward: 4 / 8 / 12 / 16 / 32 branches 1732 / 1265 /
+    // 1171 / 1143 / 1158 us); large scenes fill the GPU by themselves and
+    // compete for the L2 (12 scenes of 128^2-1024^2, forward and backward: 4071 /
+    // 4122 / 4209 / 4209 / 4207).  The line lies at a mean of 256^2 pixels.
+    const int naux = ctx->soff[ctx->nscenes] <= (long long)ctx->nscenes * 256 * 256 ? 16 : 8;
+    static_assert(hrc_ctx::kAux >= 16, "streams for every branch");
     auto enqueue = [&](cudaStream_t st, int *n, Recorder *) {
         Recorder off;   // per-launch timing is not recorded across streams
         cudaError_t err = cudaMemsetAsync(ctx->d_status, 0, sizeof(int), st);
         if (err == cudaSuccess) err = cudaEventRecord(ctx->ev_fork, st);
-        for (int k = 0; k < hrc_ctx::kAux && err == cudaSuccess; ++k) err = cudaStreamWaitEvent(ctx->aux[k], ctx->ev_fork, 0);
+        for (int k = 0; k < naux && err == cudaSuccess; ++k) err = cudaStreamWaitEvent(ctx->aux[k], ctx->ev_fork, 0);
         for (int idx = 0; idx < ctx->nscenes && err == cudaSuccess; ++idx) {
             const int i = ctx->by_size[idx];
-            cudaStream_t as = ctx->aux[idx % hrc_ctx::kAux];
+            cudaStream_t as = ctx->aux[idx % naux];
             const Plan &pl = ctx->bplans[i];
             const float *ei = (const float *)e + ctx->eoff[i], *si = (const float *)s + ctx->soff[i];
             if (mode == 0)
@@ -1755,7 +1763,7 @@ hrc_status run_batched_chains(hrc_ctx *ctx, int mode, const void *e, const void 
                 err = launch_backward(pl, ctx->rt, ei, si, (const float *)gF + ctx->eoff[i], (float *)ge + ctx->eoff[i],
                                       (float *)gs + ctx->soff[i], mode == 2, as, n, &off);
         }
-        for (int k = 0; k < hrc_ctx::kAux && err == cudaSuccess; ++k) {
+        for (int k = 0; k < naux && err == cudaSuccess; ++k) {
             err = cudaEventRecord(ctx->ev_join[k], ctx->aux[k]);
             if (err == cudaSuccess) err = cudaStreamWaitEvent(st, ctx->ev_join[k], 0);
         }
