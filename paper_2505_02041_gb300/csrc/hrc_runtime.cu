@@ -1391,7 +1391,6 @@ hrc_status hrc_reserve_bounces(hrc_ctx *ctx, int max_bounces) {
     else cudaDeviceSynchronize();
     clear_graphs(ctx);   // graphs may hold the old buffers
     cudaFree(ctx->bounce_buf);
-    cudaFree(ctx->env_tab);
     ctx->bounce_buf = nullptr;
     ctx->bounce_cap = 0;
     ctx->have_bounce = false;

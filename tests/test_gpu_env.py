@@ -158,6 +158,20 @@ def test_env_removed_and_host_entry():
     assert torch.equal(h.forward(ed, sd), F0)
 
 
+def test_env_map_survives_reserving_bounces():
+    """Reserving bounce buffers after the map was set leaves the map's tables
+    in place: the fluence matches the oracle with the map."""
+    require_gpu()
+    from paper_2505_02041_gb300 import HRC
+    e, s = scenes.random_scene(37, 23, 2, 41)
+    env = _env(2, 16, 41)
+    h = HRC(37, 23, 2)
+    h.set_environment(to_dev(env))
+    h.reserve_bounces(2)
+    F = h.forward(to_dev(e), to_dev(s)).cpu().numpy()
+    assert_fp32(F, oracle.fluence(e, s, env=env))
+
+
 def test_env_full_size_workload():
     """The 1024^2 three-channel workload under a sky-like map (bright above,
     dim below), autotuned launch configuration, against the oracle."""
