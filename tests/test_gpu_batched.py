@@ -149,6 +149,26 @@ def test_batched_schedules_match_persistent(precision):
         b.set_backward_recompute(False)
 
 
+@pytest.mark.parametrize("last", [(31, 40), (1200, 1100)])
+def test_batched_chains_on_either_branch_count(last):
+    """18 scenes (more than the branches of either count) whose mean size lies
+    below and above the line between 16 and 8 branches: schedule 1 gives the
+    persistent schedule's results to fp32 rounding."""
+    require_gpu()
+    from paper_2505_02041_gb300 import BatchedHRC
+    sizes = [(24, 24 + i) for i in range(17)] + [last]
+    es, ss = zip(*(map(torch.from_numpy, scenes.random_scene(w, h, 1, 50 + i)) for i, (w, h) in enumerate(sizes)))
+    b = BatchedHRC(sizes, 1)
+    e, s = b.pack(list(es), list(ss))
+    gF = torch.ones(e.numel(), device="cuda")
+    ref = [b.forward(e, s).clone()] + [t.clone() for t in b.backward(gF)]
+    b.tune(0, 0, 1)
+    got = [b.forward(e, s)] + list(b.backward(gF))
+    b.sync()
+    for x, y in zip(got, ref):
+        assert err_max(x.cpu().numpy(), y.cpu().numpy()) <= 1e-5
+
+
 def test_small_scene_batch_matches_single_and_oracle():
     """The benchmark's small-scene batch: 256 scenes of 64^2 .. 256^2 (C = 3,
     bf16 intervals), tuned as the benchmark tunes it.  One scene of each size:
