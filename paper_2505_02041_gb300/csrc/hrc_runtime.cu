@@ -1711,15 +1711,20 @@ hrc_status build_batched_plans(hrc_ctx *ctx, int prec) {
         ctx->bplans[i].arena = ctx->arena;
         ctx->bplans[i].solo = ctx->nscenes == 1;
         ctx->bplans[i].sched = 0;
-        ctx->bplans[i].mgroups = 1;
         ctx->bplans[i].mthreads = 128;
-        ctx->bplans[i].vmajor = 0;
-        // per-scene chains (schedule 1): the launch configuration the
-        // single-scene autotuner picks at most sizes: four v per thread in the
-        // merge up, and bulk-copy staging of the merge down in the 16-bit
-        // precisions
+        // Per-scene chains (schedule 1).  Four v per thread in the merge up, and
+        // adjacent v-blocks from 384^2 pixels on as in own_config (forward, us,
+        // off / on: 3 scenes of 2048^2 fp32 6140 / 5909, bf16 5101 / 5013; 6 of
+        // 1024^2 fp32 2782 / 2756).  Merge-down loads per thread, but bulk staging
+        // for 16-bit scenes between 384^2 and 768^2 pixels (bf16, C = 3, forward,
+        // us, per thread / bulk: 96 scenes of 64^2-256^2 1306 / 1385, 32 of 256^2
+        // 789 / 829, 16 of 512^2 1462 / 1442, 6 of 1024^2 2300 / 2363, 3 of 2048^2
+        // 5101 / 5188; fp32 16 of 512^2 1704 / 1996).
+        const long long px = (long long)ctx->Ws[i] * ctx->Hs[i];
+        const bool narrow = prec == P_FP16 || prec == P_BF16;
         ctx->bplans[i].mgroups = 4;
-        ctx->bplans[i].mdown = (prec == P_FP16 || prec == P_BF16) ? 1 : 0;
+        ctx->bplans[i].vmajor = px >= 384LL * 384 && 4LL * (ctx->Ws[i] + ctx->Hs[i]) <= 65535;
+        ctx->bplans[i].mdown = narrow && px >= 384LL * 384 && px < 768LL * 768;
         ctx->bplans[i].status = ctx->d_status;
     }
     if (off > ctx->arena_bytes) return fail(ctx, HRC_ENOMEM, "batched layout exceeds the arena");
