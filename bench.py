@@ -913,7 +913,7 @@ def bench_batched(args, dev, sizes, seed0):
            "launches_per_pass": {"forward": n_fwd, "backward": n_bwd},
            "schedule": ("persistent: trace / adjoint trace of all scenes as tile launches, the merge cascade "
                         "of all scenes in one persistent launch" if best[0] == 0 else
-                        "per-scene launch chains on 8 parallel graph branches"),
+                        "per-scene launch chains on parallel graph branches"),
            "autotune_ms": {f"sched{k[0]}_bpsm{k[1]}_order{k[2]}": v for k, v in tune.items()},
            "timed_batches": n}
     b.close()
