@@ -465,6 +465,13 @@ __device__ __forceinline__ void merge_down_entry(const Plan &pl, int q, int n, i
         // four consecutive v (v a multiple of 4, n >= 1): one 4-wide access
         // per plane and row; a far run whose even offset is not a multiple
         // of 4, or that crosses the grid edge, is read as two pairs
+        // Far entries of NB channels per range test: all of them, but two at a
+        // time at C = 4, where four take 103 registers (fp32; 128 with spills in
+        // fp64) against 64 (merge down, us, four / two: 1024^2 fp32 329 / 309,
+        // bf16 291 / 251; whole forward of 96 batched scenes of 64^2-256^2 fp32
+        // 1696 / 1409, which took 1582 with a test per channel).  With a map
+        // four are the faster form (1024^2 fp32 346 against 387 one at a time).
+        constexpr int NB = C == 4 && !ENV ? 2 : C;
         if (x & 1) {   // Eq. 14
             TLevel<P, C> Tn(pl, q, n);
             const int xq = (x + 1) >> 1;
@@ -477,14 +484,18 @@ __device__ __forceinline__ void merge_down_entry(const Plan &pl, int q, int n, i
                 const A Aj = sg == 0 ? Ap : Am;
                 Iv<P, C> t[4];
                 Tn.load4(x, kk, v, t);
-                A r[C][4], ev[C];
 #pragma unroll
-                for (int c = 0; c < C; ++c) ev[c] = renv<P, C, ENV>(pl, q, n + 1, j, c);
-                rows4<C>(rq_ok, R1.base + R1.idx(rq_ok ? xq : 0, rq_ok ? j : 0, 0, 0), g.Vs, v + 2 * kk - s, g.V, ev, r);
+                for (int c0 = 0; c0 < C; c0 += NB) {
+                    A r[NB][4], ev[NB];
 #pragma unroll
-                for (int c = 0; c < C; ++c)
+                    for (int c = 0; c < NB; ++c) ev[c] = renv<P, C, ENV>(pl, q, n + 1, j, c0 + c);
+                    rows4<NB>(rq_ok, R1.base + R1.idx(rq_ok ? xq : 0, rq_ok ? j : 0, c0, 0), g.Vs, v + 2 * kk - s, g.V, ev, r);
 #pragma unroll
-                    for (int l = 0; l < 4; ++l) acc[l][c] += fma(Aj, t[l].L[c], t[l].trans() * r[c][l]);
+                    for (int c = 0; c < NB; ++c)
+#pragma unroll
+                        for (int l = 0; l < 4; ++l)
+                            acc[l][c0 + c] += fma(Aj, t[l].L[c0 + c], t[l].trans() * r[c][l]);
+                }
             }
         } else {       // Eqs. 15-17
             TLevel<P, C> T1(pl, q, n + 1);
@@ -498,22 +509,27 @@ __device__ __forceinline__ void merge_down_entry(const Plan &pl, int q, int n, i
                 const A Aj = sg == 0 ? Ap : Am;
                 Iv<P, C> t[4];
                 T1.load4(x2, kk, v, t);
-                A r0[C][4], r1[C][4], ev[C];
 #pragma unroll
-                for (int c = 0; c < C; ++c) ev[c] = renv<P, C, ENV>(pl, q, n + 1, j, c);
-                if (!top) {
+                for (int c0 = 0; c0 < C; c0 += NB) {
+                    A r0[NB][4], r1[NB][4], ev[NB];
 #pragma unroll
-                    for (int c = 0; c < C; ++c) R1.load4(x2, j, c, v, r0[c]);
-                } else {
+                    for (int c = 0; c < NB; ++c) ev[c] = renv<P, C, ENV>(pl, q, n + 1, j, c0 + c);
+                    if (!top) {
 #pragma unroll
-                    for (int c = 0; c < C; ++c) r0[c][0] = r0[c][1] = r0[c][2] = r0[c][3] = ev[c];
+                        for (int c = 0; c < NB; ++c) R1.load4(x2, j, c0 + c, v, r0[c]);
+                    } else {
+#pragma unroll
+                        for (int c = 0; c < NB; ++c) r0[c][0] = r0[c][1] = r0[c][2] = r0[c][3] = ev[c];
+                    }
+                    rows4<NB>(r1_ok, R1.base + R1.idx(r1_ok ? x2 + 1 : 0, r1_ok ? j : 0, c0, 0), g.Vs,
+                              v + 2 * kk - 2 * s, g.V, ev, r1);
+#pragma unroll
+                    for (int c = 0; c < NB; ++c)
+#pragma unroll
+                        for (int l = 0; l < 4; ++l)
+                            acc[l][c0 + c] +=
+                                A(0.5) * (r0[c][l] + fma(Aj, t[l].L[c0 + c], t[l].trans() * r1[c][l]));
                 }
-                rows4<C>(r1_ok, R1.base + R1.idx(r1_ok ? x2 + 1 : 0, r1_ok ? j : 0, 0, 0), g.Vs, v + 2 * kk - 2 * s, g.V, ev, r1);
-#pragma unroll
-                for (int c = 0; c < C; ++c)
-#pragma unroll
-                    for (int l = 0; l < 4; ++l)
-                        acc[l][c] += A(0.5) * (r0[c][l] + fma(Aj, t[l].L[c], t[l].trans() * r1[c][l]));
             }
         }
         return;
@@ -809,6 +825,10 @@ __device__ __forceinline__ void r0_pair_add(const Plan &pl, int q, int x, int v,
     const bool top = g.N <= 1;                  // R_1 is R_N: 0, or the environment map
     const A Ap = arc<P>(pl, 1, 1), Am = arc<P>(pl, 1, 0);
     const uint64_t pol = l2_evict_first();      // T rows: read once from HBM
+    // channels per range test (see merge_down_entry): four take 74 registers and
+    // up, one block of 512 threads per SM (fp32, us, four / two: 512^2 20.3 / 16.3,
+    // 1024^2 56.8 / 49.1); the 16-bit form without a map fits 64
+    constexpr int NB = C == 4 && (ENV || sizeof(typename Prec<P>::SL) > 2) ? 2 : C;
     A acc[2][C];
 #pragma unroll
     for (int c = 0; c < C; ++c) acc[0][c] = acc[1][c] = A(0);
@@ -824,25 +844,28 @@ __device__ __forceinline__ void r0_pair_add(const Plan &pl, int q, int x, int v,
             T0.load2_ef(x, j, v, pol, t0, t1);
             const A tr0 = t0.trans(), tr1 = t1.trans();
             const int vq = v + 2 * j - 1;       // odd
-            A r0[C], r1[C], other;              // each range tested once for all channels (see rows4)
-            if (rq_ok && vq >= 0 && vq < g.V) {
 #pragma unroll
-                for (int c = 0; c < C; ++c) R1.load2(xq, j, c, vq - 1, other, r0[c]);
-            } else {
+            for (int c0 = 0; c0 < C; c0 += NB) {
+                A r0[NB], r1[NB], other;        // each range tested once for NB channels (see rows4)
+                if (rq_ok && vq >= 0 && vq < g.V) {
 #pragma unroll
-                for (int c = 0; c < C; ++c) r0[c] = renv<P, C, ENV>(pl, q, 1, j, c);
-            }
-            if (rq_ok && vq + 1 < g.V) {
+                    for (int c = 0; c < NB; ++c) R1.load2(xq, j, c0 + c, vq - 1, other, r0[c]);
+                } else {
 #pragma unroll
-                for (int c = 0; c < C; ++c) R1.load2(xq, j, c, vq + 1, r1[c], other);
-            } else {
+                    for (int c = 0; c < NB; ++c) r0[c] = renv<P, C, ENV>(pl, q, 1, j, c0 + c);
+                }
+                if (rq_ok && vq + 1 < g.V) {
 #pragma unroll
-                for (int c = 0; c < C; ++c) r1[c] = renv<P, C, ENV>(pl, q, 1, j, c);
-            }
+                    for (int c = 0; c < NB; ++c) R1.load2(xq, j, c0 + c, vq + 1, r1[c], other);
+                } else {
 #pragma unroll
-            for (int c = 0; c < C; ++c) {
-                acc[0][c] += fma(Aj, t0.L[c], tr0 * r0[c]);
-                acc[1][c] += fma(Aj, t1.L[c], tr1 * r1[c]);
+                    for (int c = 0; c < NB; ++c) r1[c] = renv<P, C, ENV>(pl, q, 1, j, c0 + c);
+                }
+#pragma unroll
+                for (int c = 0; c < NB; ++c) {
+                    acc[0][c0 + c] += fma(Aj, t0.L[c0 + c], tr0 * r0[c]);
+                    acc[1][c0 + c] += fma(Aj, t1.L[c0 + c], tr1 * r1[c]);
+                }
             }
         }
     } else {                                    // Eqs. 15-17 at n = 0: k = 2, 0 and j = 1, 0
@@ -857,29 +880,32 @@ __device__ __forceinline__ void r0_pair_add(const Plan &pl, int q, int x, int v,
             T1.load2_ef(x2, 2 * j, v, pol, t0, t1);
             const A tr0 = t0.trans(), tr1 = t1.trans();
             const int vq = v + 4 * j - 2;       // even
-            A n0[C], n1[C], f0[C], f1[C];
-            if (!top) {
 #pragma unroll
-                for (int c = 0; c < C; ++c) R1.load2(x2, j, c, v, n0[c], n1[c]);
-            } else {
+            for (int c0 = 0; c0 < C; c0 += NB) {
+                A n0[NB], n1[NB], f0[NB], f1[NB];
+                if (!top) {
 #pragma unroll
-                for (int c = 0; c < C; ++c) n0[c] = n1[c] = renv<P, C, ENV>(pl, q, 1, j, c);
-            }
-            if (r1_ok && vq >= 0 && vq < g.V) {
+                    for (int c = 0; c < NB; ++c) R1.load2(x2, j, c0 + c, v, n0[c], n1[c]);
+                } else {
 #pragma unroll
-                for (int c = 0; c < C; ++c) R1.load2(x2 + 1, j, c, vq, f0[c], f1[c]);
-                if (vq + 1 >= g.V) {
-#pragma unroll
-                    for (int c = 0; c < C; ++c) f1[c] = renv<P, C, ENV>(pl, q, 1, j, c);
+                    for (int c = 0; c < NB; ++c) n0[c] = n1[c] = renv<P, C, ENV>(pl, q, 1, j, c0 + c);
                 }
-            } else {
+                if (r1_ok && vq >= 0 && vq < g.V) {
 #pragma unroll
-                for (int c = 0; c < C; ++c) f0[c] = f1[c] = renv<P, C, ENV>(pl, q, 1, j, c);
-            }
+                    for (int c = 0; c < NB; ++c) R1.load2(x2 + 1, j, c0 + c, vq, f0[c], f1[c]);
+                    if (vq + 1 >= g.V) {
 #pragma unroll
-            for (int c = 0; c < C; ++c) {
-                acc[0][c] += A(0.5) * (n0[c] + fma(Aj, t0.L[c], tr0 * f0[c]));
-                acc[1][c] += A(0.5) * (n1[c] + fma(Aj, t1.L[c], tr1 * f1[c]));
+                        for (int c = 0; c < NB; ++c) f1[c] = renv<P, C, ENV>(pl, q, 1, j, c0 + c);
+                    }
+                } else {
+#pragma unroll
+                    for (int c = 0; c < NB; ++c) f0[c] = f1[c] = renv<P, C, ENV>(pl, q, 1, j, c0 + c);
+                }
+#pragma unroll
+                for (int c = 0; c < NB; ++c) {
+                    acc[0][c0 + c] += A(0.5) * (n0[c] + fma(Aj, t0.L[c0 + c], tr0 * f0[c]));
+                    acc[1][c0 + c] += A(0.5) * (n1[c] + fma(Aj, t1.L[c0 + c], tr1 * f1[c]));
+                }
             }
         }
     }

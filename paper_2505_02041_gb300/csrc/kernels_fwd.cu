@@ -68,8 +68,10 @@ __global__ void __launch_bounds__(128) k_merge_down_bulk(Plan pl, RowSplit rs, i
     body_merge_down_bulk<P, C, ENV>(pl, rs, n, row, vb, smem, bar);
 }
 
+// (two blocks of 512 threads per SM: the 16-bit form with a map at C = 3 would
+// take 86 registers and leave one; 512^2 bf16 whole frame 123.7 / 114.9 us)
 template <int P, int C, class OUT, bool ENV>
-__global__ void __launch_bounds__(512) k_fluence(Plan pl, OUT *__restrict__ F) {
+__global__ void __launch_bounds__(512, ENV && C == 3 && P != P_FP32 && P != P_FP64 ? 2 : 0) k_fluence(Plan pl, OUT *__restrict__ F) {
     __shared__ __align__(16) unsigned char smem[fluence_smem<P, C>()];
     body_fluence<P, C, OUT, ENV>(pl, F, blockIdx.x, blockIdx.y, smem);
 }

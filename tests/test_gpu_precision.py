@@ -129,3 +129,33 @@ def test_reduced_precision_large_grid_forms(prec, C, with_env):
     pr = np.max(np.abs(F - Fr)[lit] / np.abs(Fr)[lit])
     print(f"640x960 C={C} {prec} env={with_env}: err_max={em:.3e} relL2={l2:.3e} pixel-relative={pr:.3e}")
     assert em <= BOUNDS[prec][0] and l2 <= BOUNDS[prec][1] and pr <= BOUNDS[prec][2]
+
+
+@pytest.mark.parametrize("W,H,with_env", [(70, 53, False), (300, 261, False), (70, 53, True), (257, 131, True)])
+def test_four_channel_forms(W, H, with_env):
+    """At C = 4 the merge down and the fluence sum test the ranges of two
+    channels at a time: bit for bit the same as the bulk-staged and persistent
+    forms in every storage precision, and in fp64 equal to the oracle to
+    rounding, with odd extents, with and without a map."""
+    require_gpu()
+    from paper_2505_02041_gb300 import HRC
+    e, s = scenes.random_scene(W, H, 4, 90)
+    env = _env(4, 40, 91) if with_env else None
+    ed, sd = to_dev(e), to_dev(s)
+    for prec in ("fp32", "fp16", "bf16"):
+        h = HRC(W, H, 4, 0, prec)
+        if with_env:
+            h.set_environment(to_dev(env))
+        h.set_launch_config(0, 4, 128, 0, 0)
+        F0 = h.forward(ed, sd).clone()
+        for mdown in (1, 2):
+            h.set_launch_config(0, 4, 128, 0, mdown)
+            F = h.forward(ed, sd)
+            h.sync()
+            assert torch.equal(F, F0), (prec, mdown)
+    h = HRC(W, H, 4, 0, "fp64")
+    if with_env:
+        h.set_environment(to_dev(env))
+    e, s = e.astype(np.float64), s.astype(np.float64)
+    F = h.forward(to_dev(e, torch.float64), to_dev(s, torch.float64)).cpu().numpy()
+    assert err_max(F, oracle.fluence(e, s, env=env)) <= 1e-10
