@@ -445,10 +445,18 @@ __device__ __forceinline__ void body_merge_up4(const Plan &pl, const RowSplit &r
     Tn.store4(x, k, v, out);
 }
 
+// Channels per range test of merge_down_entry's quads: all, but two at a time at
+// C = 4, where four take 103 registers (fp32; 128 with spills in fp64) against
+// 64 (merge down, us, four / two: 1024^2 fp32 329 / 309, bf16 291 / 251; whole
+// forward of 96 batched scenes of 64^2-256^2 fp32 1696 / 1409, which took 1582
+// with a test per channel).  With a map four are the faster form (1024^2 fp32
+// 346 against 387 one at a time), and on small single grids (launch_forward).
+__host__ __device__ constexpr int range_channels(int C, bool env) { return C == 4 && !env ? 2 : C; }
+
 // R_n(p, i) = F_+ + F_-, p = (x 2^n, v), i = ip + 1/2, j_+ = 2ip+1, j_- = 2ip,
 // for v .. v+E-1 of column x >= 1 of frame q (E = 2: all neighbour offsets
 // even, n >= 1).
-template <int P, int C, int E, bool ENV = false>
+template <int P, int C, int E, bool ENV = false, int NB = range_channels(C, ENV)>
 __device__ __forceinline__ void merge_down_entry(const Plan &pl, int q, int n, int x, int ip, int v,
                                                  typename Prec<P>::A (&acc)[E][C]) {
     using A = typename Prec<P>::A;
@@ -465,13 +473,6 @@ __device__ __forceinline__ void merge_down_entry(const Plan &pl, int q, int n, i
         // four consecutive v (v a multiple of 4, n >= 1): one 4-wide access
         // per plane and row; a far run whose even offset is not a multiple
         // of 4, or that crosses the grid edge, is read as two pairs
-        // Far entries of NB channels per range test: all of them, but two at a
-        // time at C = 4, where four take 103 registers (fp32; 128 with spills in
-        // fp64) against 64 (merge down, us, four / two: 1024^2 fp32 329 / 309,
-        // bf16 291 / 251; whole forward of 96 batched scenes of 64^2-256^2 fp32
-        // 1696 / 1409, which took 1582 with a test per channel).  With a map
-        // four are the faster form (1024^2 fp32 346 against 387 one at a time).
-        constexpr int NB = C == 4 && !ENV ? 2 : C;
         if (x & 1) {   // Eq. 14
             TLevel<P, C> Tn(pl, q, n);
             const int xq = (x + 1) >> 1;
@@ -612,7 +613,7 @@ __device__ __forceinline__ void merge_down_entry(const Plan &pl, int q, int n, i
 }
 
 // One row segment of R_n with four consecutive v per thread (n >= 1).
-template <int P, int C, bool ENV = false>
+template <int P, int C, bool ENV, int NB = range_channels(C, ENV)>
 __device__ __forceinline__ void body_merge_down4(const Plan &pl, const RowSplit &rs, int n, long long bx, int by) {
     using A = typename Prec<P>::A;
     int local;
@@ -624,7 +625,7 @@ __device__ __forceinline__ void body_merge_down4(const Plan &pl, const RowSplit 
     local += I;
     const int x = local >> n, ip = local & (I - 1);
     A acc[4][C];
-    merge_down_entry<P, C, 4, ENV>(pl, q, n, x, ip, v, acc);
+    merge_down_entry<P, C, 4, ENV, NB>(pl, q, n, x, ip, v, acc);
     RLevel<P, C> Rn(pl, q, n);
 #pragma unroll
     for (int c = 0; c < C; ++c) {
@@ -804,12 +805,19 @@ __device__ __forceinline__ void body_merge_down_bulk(const Plan &pl, const RowSp
 }
 
 
+// Channels per range test of r0_pair_add (see range_channels): four take 74
+// registers and up, one block of 512 threads per SM; the 16-bit form without a
+// map fits 64.
+template <int P, int C, bool ENV> constexpr int fluence_channels() {
+    return C == 4 && (ENV || sizeof(typename Prec<P>::SL) > 2) ? 2 : C;
+}
+
 // R_0^q(x, 0, v) and R_0^q(x, 0, v + 1) (v even) added to a[0] / a[1]: the
 // n = 0 case of merge_down_entry for a pair of v, with the same arithmetic
 // per entry.  At odd x the far run starts at the odd offset v -+ 1 and is
 // read as the aligned pairs on either side of it; v + 1 may lie past V
 // (inside the padded row): that entry is computed and never used.
-template <int P, int C, bool ENV>
+template <int P, int C, bool ENV, int NB>
 __device__ __forceinline__ void r0_pair_add(const Plan &pl, int q, int x, int v, typename Prec<P>::A (&a)[2][C]) {
     using A = typename Prec<P>::A;
     const QuadGeom &g = pl.q[q];
@@ -825,10 +833,6 @@ __device__ __forceinline__ void r0_pair_add(const Plan &pl, int q, int x, int v,
     const bool top = g.N <= 1;                  // R_1 is R_N: 0, or the environment map
     const A Ap = arc<P>(pl, 1, 1), Am = arc<P>(pl, 1, 0);
     const uint64_t pol = l2_evict_first();      // T rows: read once from HBM
-    // channels per range test (see merge_down_entry): four take 74 registers and
-    // up, one block of 512 threads per SM (fp32, us, four / two: 512^2 20.3 / 16.3,
-    // 1024^2 56.8 / 49.1); the 16-bit form without a map fits 64
-    constexpr int NB = C == 4 && (ENV || sizeof(typename Prec<P>::SL) > 2) ? 2 : C;
     A acc[2][C];
 #pragma unroll
     for (int c = 0; c < C; ++c) acc[0][c] = acc[1][c] = A(0);
@@ -929,7 +933,7 @@ __device__ __forceinline__ void r0_pair_add(const Plan &pl, int q, int x, int v,
 template <int P, int C>
 constexpr size_t fluence_smem() { return sizeof(typename Prec<P>::A) * C * 32 * 33; }
 
-template <int P, int C, class OUT, bool ENV = false>
+template <int P, int C, class OUT, bool ENV = false, int NB = fluence_channels<P, C, ENV>()>
 __device__ __forceinline__ void body_fluence(const Plan &pl, OUT *__restrict__ F, int bx, int by, unsigned char *smem) {
     using A = typename Prec<P>::A;
     A (*tile)[32][33] = reinterpret_cast<A (*)[32][33]>(smem);   // [C][y][x] of the tile
@@ -942,7 +946,7 @@ __device__ __forceinline__ void body_fluence(const Plan &pl, OUT *__restrict__ F
     auto add_frame = [&](int q, int x, int y, A (&a)[2][C]) {
         int u, v;
         image_to_frame(q, W, H, x, y, u, v);
-        r0_pair_add<P, C, ENV>(pl, q, u + 1, v, a);
+        r0_pair_add<P, C, ENV, NB>(pl, q, u + 1, v, a);
     };
     for (int p = warp; p < 16; p += nw) {       // q0, q1: pixels (x, y), (x, y + 1)
         const int ca = line(p), y = y0 + 2 * hl;

@@ -2,6 +2,7 @@
 // the bodies in fwd_bodies.cuh) and the forward launch sequence.
 #include <cudaTypedefs.h>
 #include <cstring>
+#include <type_traits>
 
 #include "bulk_copy.cuh"
 #include "fwd_bodies.cuh"
@@ -50,12 +51,12 @@ __global__ void __launch_bounds__(512) k_merge_up4(Plan pl, RowSplit rs, int n) 
     body_merge_up4<P, C>(pl, rs, n, row, vb);
 }
 
-template <int P, int C, bool ENV>
+template <int P, int C, bool ENV, int NB>
 __global__ void __launch_bounds__(512) k_merge_down4(Plan pl, RowSplit rs, int n) {
     long long row;
     int vb;
     row_block(pl, row, vb);
-    body_merge_down4<P, C, ENV>(pl, rs, n, row, vb);
+    body_merge_down4<P, C, ENV, NB>(pl, rs, n, row, vb);
 }
 
 template <int P, int C, bool ENV>
@@ -70,10 +71,10 @@ __global__ void __launch_bounds__(128) k_merge_down_bulk(Plan pl, RowSplit rs, i
 
 // (two blocks of 512 threads per SM: the 16-bit form with a map at C = 3 would
 // take 86 registers and leave one; 512^2 bf16 whole frame 123.7 / 114.9 us)
-template <int P, int C, class OUT, bool ENV>
+template <int P, int C, class OUT, bool ENV, int NB>
 __global__ void __launch_bounds__(512, ENV && C == 3 && P != P_FP32 && P != P_FP64 ? 2 : 0) k_fluence(Plan pl, OUT *__restrict__ F) {
     __shared__ __align__(16) unsigned char smem[fluence_smem<P, C>()];
-    body_fluence<P, C, OUT, ENV>(pl, F, blockIdx.x, blockIdx.y, smem);
+    body_fluence<P, C, OUT, ENV, NB>(pl, F, blockIdx.x, blockIdx.y, smem);
 }
 
 // Four pixels per thread, 128 threads, 7 blocks per SM (at most 73
@@ -300,8 +301,17 @@ static cudaError_t fwd_impl(const Plan &pl, const RayTable &rt, const void *e, c
                 else
                     k_merge_down_bulk<P, C, false><<<row_grid(pl, rs.start[4], kBV), 128, BulkMD<P, C>::bytes(), st>>>(pl, rs, n);
             } else if (n >= 1) {
-                if (env) k_merge_down4<P, C, true><<<row_grid(pl, rs.start[4], 4 * mt), mt, 0, st>>>(pl, rs, n);
-                else k_merge_down4<P, C, false><<<row_grid(pl, rs.start[4], 4 * mt), mt, 0, st>>>(pl, rs, n);
+                // C = 4: two channels per range test, but all four on single grids
+                // below 256^2, where a kernel waits for its longest chain of loads
+                // (forward, fp32, us, four / two: 64^2 30.8 / 34.9, 128^2 37.1 /
+                // 43.1, 192^2 47.3 / 49.3, 256^2 57.5 / 57.6, 384^2 98.5 / 98.5,
+                // 768^2 373 / 346; 96 batched scenes of 64^2 499 / 431)
+                constexpr int NB = range_channels(C, false);
+                const dim3 grid = row_grid(pl, rs.start[4], 4 * mt);
+                if (env) k_merge_down4<P, C, true, C><<<grid, mt, 0, st>>>(pl, rs, n);
+                else if (pl.solo && (long long)pl.W * pl.H < 256LL * 256)
+                    k_merge_down4<P, C, false, C><<<grid, mt, 0, st>>>(pl, rs, n);
+                else k_merge_down4<P, C, false, NB><<<grid, mt, 0, st>>>(pl, rs, n);
             } else {
                 const int ts = 2 * mt > 512 ? 512 : 2 * mt;   // single v per thread at level 0
                 if (env) k_merge_down<P, C, false, true><<<row_grid(pl, rs.start[4], ts), ts, 0, st>>>(pl, rs, n);
@@ -337,20 +347,24 @@ static cudaError_t fwd_impl(const Plan &pl, const RayTable &rt, const void *e, c
         // 16-bit radiances is only a 4-byte access.
         const long long tiles = (long long)grid.x * grid.y;
         const int ft = tiles < 600 ? 512 : 256;
-        if constexpr (P == P_FP64) {
-            if (env) k_fluence<P, C, double, true><<<grid, ft, 0, st>>>(pl, (double *)F);
-            else k_fluence<P, C, double, false><<<grid, ft, 0, st>>>(pl, (double *)F);
-        } else if constexpr (P == P_FP16 || P == P_BF16) {
-            if (tiles >= 600) {
+        using OUT = typename std::conditional<P == P_FP64, double, float>::type;
+        // C = 4: all four channels per range test while a block has its SM to
+        // itself (152 tiles), else two, so that two fit (fp32, whole forward, us,
+        // four / two: 64^2 28.8 / 30.9, 250^2 61.6 / 62.5; fluence sum alone: 512^2
+        // 20.3 / 16.3, 1024^2 56.8 / 49.1)
+        constexpr int NBE = fluence_channels<P, C, true>(), NB0 = fluence_channels<P, C, false>();
+        const bool wide = pl.solo && tiles <= 152;
+        if ((P == P_FP16 || P == P_BF16) && tiles >= 600) {
+            if constexpr (P == P_FP16 || P == P_BF16) {
                 if (env) k_fluence4<P, C, float, true><<<grid, 128, 0, st>>>(pl, (float *)F);
                 else k_fluence4<P, C, float, false><<<grid, 128, 0, st>>>(pl, (float *)F);
-            } else {
-                if (env) k_fluence<P, C, float, true><<<grid, ft, 0, st>>>(pl, (float *)F);
-                else k_fluence<P, C, float, false><<<grid, ft, 0, st>>>(pl, (float *)F);
             }
+        } else if (env) {
+            if (wide) k_fluence<P, C, OUT, true, C><<<grid, ft, 0, st>>>(pl, (OUT *)F);
+            else k_fluence<P, C, OUT, true, NBE><<<grid, ft, 0, st>>>(pl, (OUT *)F);
         } else {
-            if (env) k_fluence<P, C, float, true><<<grid, ft, 0, st>>>(pl, (float *)F);
-            else k_fluence<P, C, float, false><<<grid, ft, 0, st>>>(pl, (float *)F);
+            if (wide) k_fluence<P, C, OUT, false, C><<<grid, ft, 0, st>>>(pl, (OUT *)F);
+            else k_fluence<P, C, OUT, false, NB0><<<grid, ft, 0, st>>>(pl, (OUT *)F);
         }
         rec->end();
         ++*launches;

@@ -131,12 +131,16 @@ def test_reduced_precision_large_grid_forms(prec, C, with_env):
     assert em <= BOUNDS[prec][0] and l2 <= BOUNDS[prec][1] and pr <= BOUNDS[prec][2]
 
 
-@pytest.mark.parametrize("W,H,with_env", [(70, 53, False), (300, 261, False), (70, 53, True), (257, 131, True)])
+@pytest.mark.parametrize("W,H,with_env", [
+    (70, 53, False), (255, 257, False), (256, 257, False), (300, 261, False), (417, 421, False), (70, 53, True), (257, 131, True),
+    (417, 421, True),
+])
 def test_four_channel_forms(W, H, with_env):
-    """At C = 4 the merge down and the fluence sum test the ranges of two
-    channels at a time: bit for bit the same as the bulk-staged and persistent
-    forms in every storage precision, and in fp64 equal to the oracle to
-    rounding, with odd extents, with and without a map."""
+    """C = 4 tests the ranges of two channels at a time in the merge down (single
+    grids from 256^2 pixels) and the fluence sum (from 153 tiles), of all four
+    below: on either side of both lines bit for bit the same as the bulk-staged
+    and persistent forms in every storage precision, and in fp64 equal to the
+    oracle to rounding, with odd extents, with and without a map."""
     require_gpu()
     from paper_2505_02041_gb300 import HRC
     e, s = scenes.random_scene(W, H, 4, 90)
