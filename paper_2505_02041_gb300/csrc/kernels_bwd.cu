@@ -45,7 +45,7 @@ __global__ void __launch_bounds__(512) k_adj_T0(Plan pl, RowSplitB rs) {
 // test per channel the merge-up reverse took 513 us instead of 387 (1024^2,
 // C = 3, fp32).  Pairs -> quads, us, C = 3 / C = 1 at 1024^2 fp32: merge-down
 // reverse 272 -> 247 / 188 -> 144, merge-up reverse 374 -> 366 / 260 -> 196;
-// bf16 C = 3: 277 -> 240, 354 -> 323.
+// bf16 C = 3: 277 -> 240, 354 -> 323.  (C = 4: see k_adj_merge_up.)
 template <int P, int C>
 __global__ void __launch_bounds__(512) k_adj_R4(Plan pl, RowSplitB rs, int n) {
     long long row;
@@ -68,6 +68,22 @@ __global__ void __launch_bounds__(512) k_adj_merge_up4(Plan pl, RowSplitB rs, in
     int vb;
     row_block_b(pl, row, vb);
     body_adj_merge_up4<P, C, ENV>(pl, rs, n, row, vb);
+}
+
+// The merge-up reverse of four channels, and of fp64, takes a pair of v per
+// thread: quads need 96-100 registers (fp64 62-128 and spills) against 40 (fp64
+// 36-100).  Quads / pairs, us: C = 4 1024^2 fp32 542 / 474, bf16 455 / 436,
+// 512^2 fp32 137 / 120, 256^2 51 / 43, whole backward of 32 batched scenes of
+// 256^2 fp32 2321 / 2013; fp64 256^2 C = 1 .. 4 70 / 65, 106 / 92, 133 / 117,
+// 166 / 143.  Single C = 4 grids below 128^2 keep the quads (64^2 18 / 20).
+template <int P, int C> constexpr bool amu_pairs() { return C == 4 || P == P_FP64; }
+
+template <int P, int C, bool ENV>
+__global__ void __launch_bounds__(512) k_adj_merge_up(Plan pl, RowSplitB rs, int n) {
+    long long row;
+    int vb;
+    row_block_b(pl, row, vb);
+    body_adj_merge_up<P, C, ENV>(pl, rs, n, row, vb);
 }
 
 template <int P, int C, class IN>
@@ -246,8 +262,26 @@ static cudaError_t bwd_impl(const Plan &pl, const RayTable &rt, const void *e, c
                 by += gTbytes(q, n - 1) + gTbytes(q, n) + bytes_T(pl, q, n - 1) + gRbytes(q, n - 1) +
                       gRbytes(q, n - 2) + bytes_R(pl, q, n - 1) + bytes_R(pl, q, n);
         rec->begin(K_ADJ_MERGE_UP, n, by);
-        if (env) k_adj_merge_up4<P, C, true><<<row_grid_b(pl, rs.start[4], 4 * mt), mt, 0, st>>>(pl, rs, n);
-        else k_adj_merge_up4<P, C, false><<<row_grid_b(pl, rs.start[4], 4 * mt), mt, 0, st>>>(pl, rs, n);
+        bool pairs = false;
+        if constexpr (amu_pairs<P, C>()) {
+            pairs = P == P_FP64 || !pl.solo || pl.W * pl.H >= 128 * 128;
+            // Grids 8 times as long as wide: every row gets the blocks of the
+            // longest, most of them empty; twice the threads halve those (fp32, us,
+            // 128 / 256 threads: 4096x64 684 / 379, 2048x128 209 / 172, 1024^2 474 /
+            // 483; fp64 C = 4 987 / 1110, so not there).
+            const int lo = pl.W < pl.H ? pl.W : pl.H, hi = pl.W < pl.H ? pl.H : pl.W;
+            const int mp = hi >= 8 * lo && hi > 2 * mt && mt <= 256 && !(P == P_FP64 && C == 4) ? 2 * mt : mt;
+            if (pairs) {
+                const dim3 grid = row_grid_b(pl, rs.start[4], 2 * mp);
+                if (env) k_adj_merge_up<P, C, true><<<grid, mp, 0, st>>>(pl, rs, n);
+                else k_adj_merge_up<P, C, false><<<grid, mp, 0, st>>>(pl, rs, n);
+            }
+        }
+        if constexpr (P != P_FP64) {
+            const dim3 grid = row_grid_b(pl, rs.start[4], 4 * mt);
+            if (!pairs && env) k_adj_merge_up4<P, C, true><<<grid, mt, 0, st>>>(pl, rs, n);
+            else if (!pairs) k_adj_merge_up4<P, C, false><<<grid, mt, 0, st>>>(pl, rs, n);
+        }
         rec->end();
         ++*launches;
     }

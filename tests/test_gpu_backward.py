@@ -235,3 +235,33 @@ def test_adjoint_quads_match_pairs(W, H, C, prec):
     b.sync()
     assert err_max(ge.cpu().numpy().reshape(-1), geb.cpu().numpy()) <= 1e-6
     assert err_max(gs.cpu().numpy().reshape(-1), gsb.cpu().numpy()) <= 1e-6
+
+
+@pytest.mark.parametrize("W,H,C,prec,with_env", [
+    (62, 61, 4, "fp32", False), (131, 127, 4, "fp32", True), (127, 129, 4, "fp32", True), (33, 517, 4, "fp32", False),
+    (521, 64, 4, "fp32", True), (62, 61, 4, "fp64", True), (41, 330, 4, "fp64", False),
+    (129, 66, 3, "fp64", False), (33, 130, 2, "fp64", True), (61, 40, 1, "fp64", False),
+])
+def test_merge_up_reverse_in_pairs(W, H, C, prec, with_env):
+    """C = 4 (from 128^2 pixels) and fp64 run the merge-up reverse with two v
+    per thread, in wider blocks where a grid is 8 times as long as wide, and
+    the steps around it with four: on either side of both lines, rows of every
+    length mod 4, with and without a map, against the oracle."""
+    require_gpu()
+    from paper_2505_02041_gb300 import HRC
+    dt = torch.float64 if prec == "fp64" else torch.float32
+    e, s = scenes.random_scene(W, H, C, 92)
+    gF = scenes.rng(93).normal(size=e.shape)
+    env = scenes.rng(94).uniform(0.0, 2.0, size=(C, 40)).astype(np.float32) if with_env else None
+    if prec == "fp32":
+        gF = gF.astype(np.float32)
+    else:
+        e, s = e.astype(np.float64), s.astype(np.float64)
+    ge_r, gs_r = oracle.fluence_adjoint(e, s, gF, env=env)
+    h = HRC(W, H, C, 0, prec)
+    if with_env:
+        h.set_environment(to_dev(env))
+    h.forward(to_dev(e, dt), to_dev(s, dt))
+    ge, gs = (t.cpu().numpy() for t in h.backward(to_dev(gF, dt)))
+    tol = 1e-4 if prec == "fp32" else 1e-10
+    assert err_max(ge, ge_r) <= tol and err_max(gs, gs_r) <= tol
