@@ -122,7 +122,8 @@ hrc_status hrc_set_schedule(hrc_ctx *ctx, int schedule);
  *   groups:   v per thread in the merge-up kernel: 1 = a pair, 2 = two pairs
  *             blockDim apart, 4 = four consecutive v;
  *   threads:  threads per block of the merge and adjoint-merge kernels
- *             (64, 128, 256 or 512);
+ *             (64, 128, 256 or 512; with 512, kernels that take four v per
+ *             thread and many registers run blocks of 256);
  *   vmajor:   grid order of those kernels: 0 = rows in gridDim.x, v-blocks
  *             in gridDim.y; 1 = the reverse (allowed while 4 (W + H) <= 65535,
  *             the gridDim.y limit for the adjoint's level-0 rows);

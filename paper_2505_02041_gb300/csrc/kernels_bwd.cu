@@ -188,7 +188,11 @@ template <int P, int C>
 static cudaError_t bwd_impl(const Plan &pl, const RayTable &rt, const void *e, const void *s, const void *gF,
                             void *ge, void *gs, bool recompute, cudaStream_t st, int *launches, Recorder *rec) {
     using IN = typename std::conditional<P == P_FP64, double, float>::type;
-    const int mt = pl.mthreads;
+    // A block of quads covers the v of a block of pairs twice as wide: 512 threads
+    // leave most of a row's threads without work and, from C = 2 on, too few
+    // blocks on an SM (backward, fp32, us, 512 / 256 threads: C = 3 1024^2 951 /
+    // 858, 256^2 133 / 107, 4096x64 845 / 650; C = 1 4096x64 505 / 544).
+    const int mt = C >= 2 && pl.mthreads > 256 ? 256 : pl.mthreads;
     const bool env = plan_has_env(pl);   // kernels compiled for an environment map
     int Nmax = 0, Nmin = pl.q[0].N;
     for (int q = 0; q < 4; ++q) {
@@ -270,7 +274,7 @@ static cudaError_t bwd_impl(const Plan &pl, const RayTable &rt, const void *e, c
             // 128 / 256 threads: 4096x64 684 / 379, 2048x128 209 / 172, 1024^2 474 /
             // 483; fp64 C = 4 987 / 1110, so not there).
             const int lo = pl.W < pl.H ? pl.W : pl.H, hi = pl.W < pl.H ? pl.H : pl.W;
-            const int mp = hi >= 8 * lo && hi > 2 * mt && mt <= 256 && !(P == P_FP64 && C == 4) ? 2 * mt : mt;
+            const int mp = hi >= 8 * lo && hi > 2 * mt && mt <= 256 && !(P == P_FP64 && C == 4) ? 2 * mt : pl.mthreads;
             if (pairs) {
                 const dim3 grid = row_grid_b(pl, rs.start[4], 2 * mp);
                 if (env) k_adj_merge_up<P, C, true><<<grid, mp, 0, st>>>(pl, rs, n);

@@ -307,6 +307,11 @@ static cudaError_t fwd_impl(const Plan &pl, const RayTable &rt, const void *e, c
                 // 43.1, 192^2 47.3 / 49.3, 256^2 57.5 / 57.6, 384^2 98.5 / 98.5,
                 // 768^2 373 / 346; 96 batched scenes of 64^2 499 / 431)
                 constexpr int NB = range_channels(C, false);
+                // At C >= 3 (fp64: 2) a quad takes 64 registers and up, so that a second
+                // block of 512 threads does not fit the SM: blocks of 256 at most
+                // (forward, C = 3 fp32, us, 512 / 256 threads: 512^2 198 / 139, 4096x64
+                // 1134 / 818)
+                const int mt = C >= (P == P_FP64 ? 2 : 3) && pl.mthreads > 256 ? 256 : pl.mthreads;
                 const dim3 grid = row_grid(pl, rs.start[4], 4 * mt);
                 if (env) k_merge_down4<P, C, true, C><<<grid, mt, 0, st>>>(pl, rs, n);
                 else if (pl.solo && (long long)pl.W * pl.H < 256LL * 256)
