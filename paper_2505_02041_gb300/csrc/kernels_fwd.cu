@@ -233,10 +233,14 @@ static cudaError_t fwd_impl(const Plan &pl, const RayTable &rt, const void *e, c
             // again, so grids that fill the GPU take whole tiles.  fp32,
             // parts 1 / 2 / 4 / 16 (trace alone, us): 64^2 13.0 / 10.4 / 9.2 /
             // 8.6, 256^2 13.2 / 11.1 / 10.7 / 17.9, 384^2 C = 3 15.4 / 14.4 /
-            // 18.0 / 34.8, 512^2 C = 3 19.1 / 22.8 / 24.7 / 53.9.  Not in a
-            // batch, whose scenes share the GPU.
+            // 18.0 / 34.8, 512^2 C = 3 19.1 / 22.8 / 24.7 / 53.9.  An fp64 tile
+            // fills an SM and takes 50 us to stage, so there is room for half as
+            // many (C = 1, parts 1 / 2 / 4 / 16: 96^2 97 / 73 / 61 / 54, 128^2 98 /
+            // 73 / 61 / 95, 192^2 97 / 73 / 62 / 185, 256^2 98 / 74 / 113 / 363, 288^2
+            // 98 / 135 / 167 / 452).  Not in a batch, whose scenes share the GPU.
             const unsigned tiles = grid.x * grid.y;
-            if (pl.solo) grid.z = tiles <= 19 ? 16 : (tiles <= 76 ? 4 : (tiles <= 152 ? 2 : 1));
+            const unsigned room = P == P_FP64 ? 152 : 304;
+            if (pl.solo) grid.z = 16 * tiles <= room ? 16 : (4 * tiles <= room ? 4 : (2 * tiles <= room ? 2 : 1));
             rec->begin(K_TRACE012, 0, by);
             CUtensorMap me, ms;
             std::memset(&me, 0, sizeof(me));

@@ -326,3 +326,14 @@ def test_trace_parts_on_grids_of_few_tiles(W, H):
     e, s = scenes.random_scene(W, H, 1, 95)
     _, F = _gpu_F(e, s)
     assert_fp32(F, oracle.fluence(e, s))
+
+
+@pytest.mark.parametrize("W,H", [(281, 30), (320, 32), (606, 60), (620, 61), (1201, 63), (1230, 64)])
+def test_trace_parts_in_fp64(W, H):
+    """In fp64 the lines lie at 9, 38 and 76 tiles: sizes on either side of each,
+    against the oracle to rounding."""
+    require_gpu()
+    e, s = (x.astype(np.float64) for x in scenes.random_scene(W, H, 1, 96))
+    from paper_2505_02041_gb300 import HRC
+    F = HRC(W, H, 1, 0, "fp64").forward(to_dev(e), to_dev(s)).cpu().numpy()
+    assert err_max(F, oracle.fluence(e, s)) <= 1e-10
