@@ -297,15 +297,19 @@ static cudaError_t bwd_impl(const Plan &pl, const RayTable &rt, const void *e, c
         // Both pairs in one launch and their sum in a second one: two launches
         // of 4.5 waves each (1024^2, 456 blocks resident) become one of 9, and
         // pair 1 no longer reads what pair 0 wrote.  While a block per tile and
-        // frame fits the GPU at once (3 blocks per SM: 2 (n0 + n1) <= 456), a
-        // tile's two frames are halved too.  Adjoint trace in all, C = 3, fp32,
+        // frame fits the GPU at once (3 blocks per SM at C <= 3, 2 at C = 4, 1 in
+        // fp64, of 152), a tile's two frames are halved too.  Adjoint trace in all, C = 3, fp32,
         // us, one pair after the other / pairs at once / frames at once:
         // 64^2 40.9 / 24.4 / 17.3, 256^2 44.0 / 30.2 / 35.9, 512^2 97 / 79 / 85,
-        // 1024^2 269 / 254 / 309, 2048^2 987 / 966 / 1216.  The planes need
-        // dL/dR_1 buffers (N >= 2 in every frame).
+        // 1024^2 269 / 254 / 309, 2048^2 987 / 966 / 1216; on either side of the
+        // lines, pairs / frames at once: fp64 C = 1 128^2 117 / 82, 144^2 118 /
+        // 145, C = 4 170 / 108, 174 / 203; C = 4 fp32 176^2 28.2 / 22.5, 200^2 34.7 /
+        // 36.5; C = 1 224^2 25.5 / 22.1, 256^2 24.5 / 28.6.  The planes need dL/dR_1
+        // buffers (N >= 2 in every frame).
         const bool all = Nmin >= 2;
         if (all) {
-            const bool one = pl.solo && n0 + n1 <= 228;   // a frame per block
+            const int room = 152 * (P == P_FP64 ? 1 : (C == 4 ? 2 : 3));
+            const bool one = pl.solo && 2 * (n0 + n1) <= room;   // a frame per block
             double by = img * (pl.C + 1) * ab * (one ? 10.0 : 5.0);   // the inputs, the planes written and read, the sums
             for (int q = 0; q < 4; ++q)
                 for (int n = 0; n <= 2; ++n) by += gTbytes(q, n);

@@ -265,3 +265,24 @@ def test_merge_up_reverse_in_pairs(W, H, C, prec, with_env):
     ge, gs = (t.cpu().numpy() for t in h.backward(to_dev(gF, dt)))
     tol = 1e-4 if prec == "fp32" else 1e-10
     assert err_max(ge, ge_r) <= tol and err_max(gs, gs_r) <= tol
+
+
+@pytest.mark.parametrize("W,H,C,prec", [
+    (123, 143, 2, "fp64"), (123, 147, 2, "fp64"), (239, 247, 1, "fp64"), (135, 255, 4, "fp32"), (159, 239, 4, "fp32"),
+    (223, 255, 3, "fp32"), (181, 289, 3, "fp32"), (181, 289, 2, "fp32"),
+])
+def test_adjoint_trace_at_its_lines(W, H, C, prec):
+    """A frame per block up to 76 tiles in fp64, 152 at C = 4 and 228 else, a pair
+    per block above: sizes next to each line (76 and 80, 152 and 155, 224 and 234
+    tiles, and fp64 far above), odd extents, against the oracle."""
+    require_gpu()
+    e, s = scenes.random_scene(W, H, C, 97)
+    gF = scenes.rng(98).normal(size=e.shape)
+    if prec == "fp64":
+        e, s = e.astype(np.float64), s.astype(np.float64)
+    else:
+        gF = gF.astype(np.float32)
+    ge_r, gs_r = oracle.fluence_adjoint(e, s, gF)
+    ge, gs = _gpu_grads(e, s, gF, prec)
+    tol = 1e-10 if prec == "fp64" else 1e-4
+    assert err_max(ge, ge_r) <= tol and err_max(gs, gs_r) <= tol
