@@ -1706,25 +1706,51 @@ hrc_status build_batched_tables(hrc_ctx *ctx) {
 hrc_status build_batched_plans(hrc_ctx *ctx, int prec) {
     size_t off = 0;
     ctx->bplans.assign(ctx->nscenes, Plan());
+    // Per-scene chains: bulk-staged merge down for the whole batch or for none of
+    // it (scenes of both forms side by side are slower than either: C = 3 bf16, 8
+    // scenes of 512-2048 a side 5245 per thread, 5348 bulk, 5579 mixed).  Bulk
+    // blocks cover 512 v and pay in 16 bits where rows fill them: `fill` is the
+    // share of their v that is used.  bf16, forward, us, per thread / bulk, one
+    // size: C = 4 320^2 1373 / 1414, 384^2 1466 / 1475, 416^2 1764 / 1686, 512^2 2014
+    // / 1925, 544^2 2890 / 3049, 640^2 2375 / 2519, 768^2 2608 / 2676, 896^2 3623 /
+    // 3597, 1024^2 3370 / 3309, 2048^2 5078 / 4811; C = 3 384^2 1081 / 1087, 416^2
+    // 1300 / 1251, 512^2 1487 / 1462, 544^2 2122 / 2260, 1024^2 2327 / 2389, 2048^2
+    // 3435 / 3483 (C = 2 alike); C = 1 512^2 801 / 819.
+    double used = 0, area = 0;
+    int vmax = 0;
+    for (int i = 0; i < ctx->nscenes; ++i) {
+        const double a = double(ctx->Ws[i]) * ctx->Hs[i];
+        for (int V : {ctx->Ws[i], ctx->Hs[i]}) {
+            used += 0.5 * a * V / (512.0 * ((V + 511) / 512));
+            vmax = std::max(vmax, V);
+        }
+        area += a;
+    }
+    const bool bulk = (prec == P_FP16 || prec == P_BF16) && ctx->C >= 2 && used >= 0.8 * area &&
+                      (ctx->C == 4 || vmax <= 512);
     for (int i = 0; i < ctx->nscenes; ++i) {
         off = build_plan(ctx->Ws[i], ctx->Hs[i], ctx->C, ctx->cascades, prec, off, ctx->bplans[i], true);
         ctx->bplans[i].arena = ctx->arena;
         ctx->bplans[i].solo = ctx->nscenes == 1;
         ctx->bplans[i].sched = 0;
-        ctx->bplans[i].mthreads = 128;
         // Per-scene chains (schedule 1).  Four v per thread in the merge up, and
         // adjacent v-blocks from 384^2 pixels on as in own_config (forward, us,
         // off / on: 3 scenes of 2048^2 fp32 6140 / 5909, bf16 5101 / 5013; 6 of
-        // 1024^2 fp32 2782 / 2756).  Merge-down loads per thread, but bulk staging
-        // for 16-bit scenes between 384^2 and 768^2 pixels (bf16, C = 3, forward,
-        // us, per thread / bulk: 96 scenes of 64^2-256^2 1306 / 1385, 32 of 256^2
-        // 789 / 829, 16 of 512^2 1462 / 1442, 6 of 1024^2 2300 / 2363, 3 of 2048^2
-        // 5101 / 5188; fp32 16 of 512^2 1704 / 1996).
+        // 1024^2 fp32 2782 / 2756) -- but not for oblong scenes of four fp32 channels
+        // (12 of 512x1024 3641 / 4377, 8 of 512-2048 a side 7854 / 10055; square
+        // 14 of 544^2 3749 / 3554).
+        // Rows of up to 256 v take blocks of 64 threads, one block per row: of 128
+        // threads with four v each at least half would have no work, and their
+        // registers keep other blocks out (C = 3, 16 branches, us, 128 / 64 threads,
+        // forward and backward: 48 of 160^2 fp32 691 / 551 and 1189 / 1045, bf16 663 /
+        // 543 and 1171 / 1028; 32 of 256^2 on 8 branches 808 / 688 and 1608 / 1518; 24
+        // of 320^2 1157 / 1249 and 2095 / 2268).
         const long long px = (long long)ctx->Ws[i] * ctx->Hs[i];
-        const bool narrow = prec == P_FP16 || prec == P_BF16;
+        ctx->bplans[i].mthreads = std::max(ctx->Ws[i], ctx->Hs[i]) <= 256 ? 64 : 128;
+        const bool oblong4 = ctx->C == 4 && prec == P_FP32 && ctx->Ws[i] != ctx->Hs[i];
         ctx->bplans[i].mgroups = 4;
-        ctx->bplans[i].vmajor = px >= 384LL * 384 && 4LL * (ctx->Ws[i] + ctx->Hs[i]) <= 65535;
-        ctx->bplans[i].mdown = narrow && px >= 384LL * 384 && px < 768LL * 768;
+        ctx->bplans[i].vmajor = px >= 384LL * 384 && 4LL * (ctx->Ws[i] + ctx->Hs[i]) <= 65535 && !oblong4;
+        ctx->bplans[i].mdown = bulk;
         ctx->bplans[i].status = ctx->d_status;
     }
     if (off > ctx->arena_bytes) return fail(ctx, HRC_ENOMEM, "batched layout exceeds the arena");
@@ -1744,12 +1770,15 @@ hrc_status build_batched_plans(hrc_ctx *ctx, int prec) {
 hrc_status run_batched_chains(hrc_ctx *ctx, int mode, const void *e, const void *s, void *F, const void *gF,
                               void *ge, void *gs, const char *where) {
     // Branches: a small scene's kernels leave most of the GPU idle and follow
-    // each other at their own latency, so more chains at once help (96 scenes
-    // of 64^2-256^2, bf16, forward: 4 / 8 / 12 / 16 / 32 branches 1732 / 1265 /
-    // 1171 / 1143 / 1158 us); large scenes fill the GPU by themselves and
-    // compete for the L2 (12 scenes of 128^2-1024^2, forward and backward: 4071 /
-    // 4122 / 4209 / 4209 / 4207).  The line lies at a mean of 256^2 pixels.
-    const int naux = ctx->soff[ctx->nscenes] <= (long long)ctx->nscenes * 256 * 256 ? 16 : 8;
+    // each other at their own latency, so more chains at once help; larger ones
+    // fill the GPU by themselves and compete for the L2.  Forward + backward, us,
+    // 8 / 16 branches, scenes of one size: C = 3 fp32 64^2 1705 / 1082, 128^2 1628 /
+    // 1422, 160^2 1675 / 1596, 192^2 1712 / 1716, 224^2 2034 / 2111, 256^2 2206 / 2310;
+    // bf16 192^2 1692 / 1633, 224^2 1939 / 1970; C = 1 fp32 224^2 1380 / 1309, 256^2
+    // 1362 / 1338, 320^2 1818 / 1863.  The line lies at a mean of 208^2 pixels, at
+    // C = 1 of 256^2.
+    const long long mean = ctx->C == 1 ? 256 * 256 : 208 * 208;
+    const int naux = ctx->soff[ctx->nscenes] <= ctx->nscenes * mean ? 16 : 8;
     static_assert(hrc_ctx::kAux >= 16, "streams for every branch");
     auto enqueue = [&](cudaStream_t st, int *n, Recorder *) {
         Recorder off;   // per-launch timing is not recorded across streams

@@ -249,3 +249,28 @@ def test_full_size_64_scene_batch_against_oracle():
         assert np.linalg.norm(Fg - Fr) <= 2e-3 * np.linalg.norm(Fr), X
     assert checked == {128, 512, 1024, 2048}
     b.close()
+
+
+@pytest.mark.parametrize("C,sizes", [
+    (2, [(449, 430), (511, 500), (470, 449)]),      # rows fill the 512-wide blocks: bulk staging
+    (3, [(449, 430), (513, 500)]),                  # a row of two blocks: per thread
+    (4, [(1021, 509), (510, 449)]),                 # bulk staging at C = 4
+    (4, [(385, 300), (130, 70)]),                   # rows that do not fill them: per thread
+    (1, [(500, 500)]),
+])
+def test_batched_chains_merge_down_forms(C, sizes):
+    """The chains stage the merge down by bulk copies for the whole batch or for
+    none of it: on either side of the rule, bf16, the forward and backward of
+    the persistent schedule to fp32 rounding."""
+    require_gpu()
+    from paper_2505_02041_gb300 import BatchedHRC
+    es, ss = zip(*(map(torch.from_numpy, scenes.random_scene(w, h, C, 70 + i)) for i, (w, h) in enumerate(sizes)))
+    b = BatchedHRC(sizes, C, precision="bf16")
+    e, s = b.pack(list(es), list(ss))
+    gF = torch.from_numpy(scenes.rng(71).normal(size=e.numel()).astype(np.float32)).cuda()
+    ref = [b.forward(e, s).clone()] + [t.clone() for t in b.backward(gF)]
+    b.tune(0, 0, 1)
+    got = [b.forward(e, s)] + list(b.backward(gF))
+    b.sync()
+    for x, y in zip(got, ref):
+        assert err_max(x.cpu().numpy(), y.cpu().numpy()) <= 1e-5
