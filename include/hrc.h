@@ -135,15 +135,15 @@ hrc_status hrc_set_schedule(hrc_ctx *ctx, int schedule);
  *             level-to-level dependencies are tracked by per-column
  *             completion counters with bounded waits; not with schedule 2).
  *             FP64 always uses 0.
- * Defaults {0, 1, 128, 0, 0}; hrc_autotune picks one.  Until a configuration
- * is set or autotuned, a context of 384^2 pixels and more runs its merge
- * kernels with groups 4 and grid order 1 (where that is allowed); the values
- * read back are the defaults all the same. */
+ * A context begins with {0, 1, 128, 0, 0}, from 384^2 pixels on with {0, 4, 128,
+ * 1, 0} (vmajor 0 where 1 is not allowed) outside FP64; hrc_autotune picks
+ * one.  A configuration that was set holds in every precision. */
 typedef struct hrc_launch_config {
     int schedule, groups, threads, vmajor, mdown;
 } hrc_launch_config;
 
-/* Read / set the launch configuration.  Setting it forgets the borrowed
+/* Read / set the launch configuration: what is read is what the context runs in
+ * its present precision, and setting that again changes nothing.  Setting it forgets the borrowed
  * forward inputs (run hrc_fluence again before hrc_fluence_backward).
  * HRC_EINVAL for a value outside the ranges above. */
 hrc_status hrc_get_launch_config(const hrc_ctx *ctx, hrc_launch_config *cfg);

@@ -178,11 +178,11 @@ struct hrc_ctx {
     int W = 0, H = 0, C = 0, cascades = 0;
     int prec = P_FP32;
     int sched = 0;
-    int mgroups = 1;
+    int mgroups = 1;             // fp32 / fp16 / bf16 (initial values: own_config)
     int mthreads = 128;
     int vmajor = 0;
     int mdown = 0;
-    bool cfg_set = false;        // a launch configuration was set or autotuned (else own_config decides)
+    int mgroups64 = 1, vmajor64 = 0;   // the same in fp64
     int device = 0;
     cudaStream_t stream = nullptr;
     RayTable rt;
@@ -345,22 +345,24 @@ cudaError_t upload_arcs(const Plan &pl, char *arena) {
     return cudaMemcpy(arena + pl.arcs_off_d, ad.data(), ad.size() * sizeof(double), cudaMemcpyHostToDevice);
 }
 
-// The plan of a pass in a context whose launch configuration nobody has set:
-// on grids of 384^2 pixels and more the merge up takes four v per thread and
-// the v-blocks of a row are adjacent in launch order, the autotuner's choice at
-// nearly every such size (forward in fp32, C = 3, us, the initial
-// configuration / this one: 512^2 113.0 / 110.9, 768^2 257.5 / 253.8, 1024^2
-// 484 / 461, 2048^2 2028 / 1888; bf16 2048^2 2046 / 1737).  Below, half the threads
-// cost more than the wider loads save (256^2: 49.2 / 49.3, C = 1 41.0 / 41.7).
-Plan own_config(const hrc_ctx *ctx, const Plan &base) {
-    Plan pl = base;
-    if (!ctx->cfg_set && (long long)ctx->W * ctx->H >= 384LL * 384 && ctx->prec != P_FP64) {
-        pl.mgroups = 4;
-        if (4LL * (ctx->W + ctx->H) <= 65535) pl.vmajor = 1;
-    }
-    return pl;
+// The launch configuration a context begins with: on grids of 384^2 pixels and
+// more the merge up takes four v per thread and the v-blocks of a row are
+// adjacent in launch order, the autotuner's choice at nearly every such size
+// (forward in fp32, C = 3, us, groups 1 and grid order 0 / this one: 512^2 113.0 /
+// 110.9, 768^2 257.5 / 253.8, 1024^2 484 / 461, 2048^2 2028 / 1888; bf16 2048^2
+// 2046 / 1737).  Below, half the threads cost more than the wider loads save
+// (256^2: 49.2 / 49.3, C = 1 41.0 / 41.7), and in fp64 they do everywhere (512^2
+// 396 / 403, 1024^2 1436 / 1447).
+void own_config(hrc_ctx *ctx) {
+    if ((long long)ctx->W * ctx->H < 384LL * 384) return;
+    ctx->mgroups = 4;
+    if (4LL * (ctx->W + ctx->H) <= 65535) ctx->vmajor = 1;
 }
-int groups_key(const hrc_ctx *ctx) { return ctx->mgroups + (ctx->cfg_set ? 16 : 0); }
+// The values of the present precision.
+int run_groups(const hrc_ctx *ctx) { return ctx->prec == P_FP64 ? ctx->mgroups64 : ctx->mgroups; }
+int run_vmajor(const hrc_ctx *ctx) { return ctx->prec == P_FP64 ? ctx->vmajor64 : ctx->vmajor; }
+// The part of a graph's key that the configuration of its kernels makes up.
+int tune_key(const hrc_ctx *ctx) { return ctx->mthreads * 8 + run_vmajor(ctx) * 4 + ctx->mdown; }
 
 // Enqueue one pass (forward or backward) on the context's stream: replay its
 // CUDA graph when one exists for these pointers, capture one otherwise.
@@ -389,8 +391,8 @@ hrc_status run_pass_key(hrc_ctx *ctx, int kind, const PassKey &pk, ENQ &&enqueue
     const bool timed = ctx->rec.on;
     const void *const *key = pk.p;
     for (auto &g : ctx->graphs) {
-        if (g.exec && g.kind == kind && g.prec == ctx->prec && g.sched == ctx->sched && g.mgroups == groups_key(ctx) &&
-            g.tune == ctx->mthreads * 8 + ctx->vmajor * 4 + ctx->mdown && g.timed == (timed ? ctx->timing_mode : 0) &&
+        if (g.exec && g.kind == kind && g.prec == ctx->prec && g.sched == ctx->sched && g.mgroups == run_groups(ctx) &&
+            g.tune == tune_key(ctx) && g.timed == (timed ? ctx->timing_mode : 0) &&
             std::memcmp(g.p, key, sizeof(pk.p)) == 0) {
             cudaError_t e = cudaGraphLaunch(g.exec, ctx->stream);
             if (e != cudaSuccess) return cuda_fail(ctx, e, where);
@@ -412,8 +414,8 @@ hrc_status run_pass_key(hrc_ctx *ctx, int kind, const PassKey &pk, ENQ &&enqueue
         mix((unsigned long long)kind);
         mix((unsigned long long)ctx->prec);
         mix((unsigned long long)ctx->sched);
-        mix((unsigned long long)groups_key(ctx));
-        mix((unsigned long long)(ctx->mthreads * 8 + ctx->vmajor * 4 + ctx->mdown));
+        mix((unsigned long long)run_groups(ctx));
+        mix((unsigned long long)tune_key(ctx));
         for (int i = 0; i < 8; ++i) mix((unsigned long long)(uintptr_t)key[i]);
         int unreplayed = 0;
         for (const auto &g : ctx->graphs) unreplayed += (g.exec && g.replays == 0) ? 1 : 0;
@@ -465,8 +467,8 @@ hrc_status run_pass_key(hrc_ctx *ctx, int kind, const PassKey &pk, ENQ &&enqueue
     slot.kind = kind;
     slot.prec = ctx->prec;
     slot.sched = ctx->sched;
-    slot.mgroups = groups_key(ctx);
-    slot.tune = ctx->mthreads * 8 + ctx->vmajor * 4 + ctx->mdown;
+    slot.mgroups = run_groups(ctx);
+    slot.tune = tune_key(ctx);
     slot.timed = timed ? ctx->timing_mode : 0;
     slot.recs = timed ? ctx->rec.recs : std::vector<Recorder::Rec>();
     std::memcpy(slot.p, key, sizeof(pk.p));
@@ -608,6 +610,7 @@ hrc_status hrc_create(int W, int H, int channels, int cascades, hrc_ctx **out) {
     hrc_ctx *ctx = new (std::nothrow) hrc_ctx();
     if (!ctx) return fail(nullptr, HRC_ENOMEM, "hrc_create: host allocation failed");
     ctx->W = W; ctx->H = H; ctx->C = channels; ctx->cascades = cascades;
+    own_config(ctx);
     ctx->rt = make_ray_table();
     cudaError_t e = cudaGetDevice(&ctx->device);
     if (e == cudaSuccess) e = prepare_device_once();
@@ -740,12 +743,25 @@ bool config_valid(const hrc_ctx *ctx, const hrc_launch_config &c) {
            !(c.vmajor && 4LL * (ctx->W + ctx->H) > 65535);
 }
 
-void apply_config(hrc_ctx *ctx, const hrc_launch_config &c) {
-    hrc_set_schedule(ctx, c.schedule);
-    ctx->mgroups = ctx->plan.mgroups = ctx->plan64.mgroups = c.groups;
+// A context's whole configuration (fp64 apart), into the context and its plans.
+struct FullConfig {
+    int sched, threads, mdown, groups, vmajor, groups64, vmajor64;
+};
+FullConfig full_config(const hrc_ctx *ctx) {
+    return {ctx->sched, ctx->mthreads, ctx->mdown, ctx->mgroups, ctx->vmajor, ctx->mgroups64, ctx->vmajor64};
+}
+void apply_full(hrc_ctx *ctx, const FullConfig &c) {
+    hrc_set_schedule(ctx, c.sched);
     ctx->mthreads = ctx->plan.mthreads = ctx->plan64.mthreads = c.threads;
-    ctx->vmajor = ctx->plan.vmajor = ctx->plan64.vmajor = c.vmajor;
     ctx->mdown = ctx->plan.mdown = ctx->plan64.mdown = c.mdown;
+    ctx->mgroups = ctx->plan.mgroups = c.groups;
+    ctx->vmajor = ctx->plan.vmajor = c.vmajor;
+    ctx->mgroups64 = ctx->plan64.mgroups = c.groups64;
+    ctx->vmajor64 = ctx->plan64.vmajor = c.vmajor64;
+}
+// A configuration set by the caller holds in every precision.
+void apply_config(hrc_ctx *ctx, const hrc_launch_config &c) {
+    apply_full(ctx, {c.schedule, c.threads, c.mdown, c.groups, c.vmajor, c.groups, c.vmajor});
 }
 }  // namespace
 
@@ -820,9 +836,9 @@ hrc_status hrc_get_cross_blur(const hrc_ctx *ctx, int *enable, float *threshold)
 hrc_status hrc_get_launch_config(const hrc_ctx *ctx, hrc_launch_config *cfg) {
     if (!ctx || !cfg) return HRC_EINVAL;
     cfg->schedule = ctx->sched;
-    cfg->groups = ctx->mgroups;
+    cfg->groups = run_groups(ctx);
     cfg->threads = ctx->mthreads;
-    cfg->vmajor = ctx->vmajor;
+    cfg->vmajor = run_vmajor(ctx);
     cfg->mdown = ctx->mdown;
     return HRC_OK;
 }
@@ -832,7 +848,6 @@ hrc_status hrc_set_launch_config(hrc_ctx *ctx, const hrc_launch_config *cfg) {
     if (ctx->batched) return fail(ctx, HRC_EINVAL, "hrc_set_launch_config: single-scene contexts only");
     if (!config_valid(ctx, *cfg)) return fail(ctx, HRC_EINVAL, "hrc_set_launch_config: value out of range");
     apply_config(ctx, *cfg);
-    ctx->cfg_set = true;
     ctx->have_fwd = false;
     for (hrc_ctx *k : ctx->chan) hrc_set_launch_config(k, cfg);
     return HRC_OK;
@@ -858,11 +873,11 @@ hrc_status hrc_autotune(hrc_ctx *ctx, float *best_ms) {
     cudaEventCreate(&a);
     cudaEventCreate(&b);
     float best = 1e30f;
+    const FullConfig before = full_config(ctx);
     hrc_launch_config best_c;
     hrc_get_launch_config(ctx, &best_c);
     const bool timing = ctx->rec.on;
     ctx->rec.on = false;
-    ctx->cfg_set = true;
     static const int kThreads[4] = {64, 128, 256, 512};
     static const int kGroups[3] = {1, 2, 4};
     for (int cand = 0; cand < 3 * 3 * 4 * 2 * 3 && st == HRC_OK; ++cand) {
@@ -884,9 +899,12 @@ hrc_status hrc_autotune(hrc_ctx *ctx, float *best_ms) {
     cudaEventDestroy(a);
     cudaEventDestroy(b);
     ctx->rec.on = timing;
-    apply_config(ctx, best_c);
     ctx->have_fwd = false;
-    if (st != HRC_OK) return st;
+    if (st != HRC_OK) {
+        apply_full(ctx, before);
+        return st;
+    }
+    apply_config(ctx, best_c);
     if (best_ms) *best_ms = best;
     return HRC_OK;
 }
@@ -939,9 +957,9 @@ hrc_status hrc_set_precision(hrc_ctx *ctx, hrc_precision prec) {
             ctx->arena64_bytes = bytes;
             p64.arena = ctx->arena64;
             p64.sched = ctx->sched;
-            p64.mgroups = ctx->mgroups;
+            p64.mgroups = ctx->mgroups64;
             p64.mthreads = ctx->mthreads;
-            p64.vmajor = ctx->vmajor;
+            p64.vmajor = ctx->vmajor64;
             p64.mdown = ctx->mdown;
             p64.status = reinterpret_cast<int *>(ctx->pctl + 8);
             ctx->plan64 = p64;
@@ -1119,16 +1137,13 @@ hrc_status hrc_set_channel_extinction(hrc_ctx *ctx, int per_channel) {
                 return fail(ctx, HRC_ENOMEM, "hrc_set_channel_extinction: staging buffers do not fit");
             }
         }
-        hrc_launch_config cfg;
-        hrc_get_launch_config(ctx, &cfg);
         for (int c = 0; c < ctx->C; ++c) {
             hrc_ctx *k = nullptr;
             hrc_status st = hrc_create(ctx->W, ctx->H, 1, ctx->cascades, &k);
             if (st == HRC_OK) ctx->chan.push_back(k);
             if (st == HRC_OK) st = hrc_set_stream(k, ctx->stream);
             if (st == HRC_OK) st = hrc_set_precision(k, (hrc_precision)ctx->prec);
-            if (st == HRC_OK) st = hrc_set_launch_config(k, &cfg);
-            if (st == HRC_OK) k->cfg_set = ctx->cfg_set;
+            if (st == HRC_OK) apply_full(k, full_config(ctx));
             if (st == HRC_OK) st = hrc_set_backward_recompute(k, ctx->bwd_recompute ? 1 : 0);
             if (st == HRC_OK && ctx->blur_buf) st = hrc_set_cross_blur(k, ctx->blur ? 1 : 0, ctx->blur_thr);
             if (st == HRC_OK && ctx->bounce_buf) st = hrc_reserve_bounces(k, ctx->bounce_cap);
@@ -1258,7 +1273,7 @@ hrc_status hrc_fluence(hrc_ctx *ctx, const float *emission, const float *sigma_t
     if (!emission || !sigma_t || !out) return fail(ctx, HRC_EINVAL, "hrc_fluence: NULL pointer");
     if (!aligned16(emission) || !aligned16(sigma_t) || !aligned16(out))
         return fail(ctx, HRC_EINVAL, "hrc_fluence: pointers must be 16-byte aligned");
-    const Plan pl = own_config(ctx, ctx->plan);
+    const Plan pl = ctx->plan;
     const RayTable *rt = &ctx->rt;
     void *Fr = ctx->blur ? ctx->blur_buf : nullptr;
     const double thr = ctx->blur_thr;
@@ -1338,7 +1353,7 @@ hrc_status hrc_fluence_backward(hrc_ctx *ctx, const float *grad_F, float *grad_e
     if (!grad_F || !grad_emission || !grad_sigma_t) return fail(ctx, HRC_EINVAL, "hrc_fluence_backward: NULL pointer");
     if (!aligned16(grad_F) || !aligned16(grad_emission) || !aligned16(grad_sigma_t))
         return fail(ctx, HRC_EINVAL, "hrc_fluence_backward: pointers must be 16-byte aligned");
-    const Plan pl = own_config(ctx, ctx->plan);
+    const Plan pl = ctx->plan;
     const RayTable *rt = &ctx->rt;
     const void *le = ctx->last_e, *ls = ctx->last_s;
     const bool rc = ctx->bwd_recompute;
@@ -1434,7 +1449,7 @@ hrc_status bounces_forward(hrc_ctx *ctx, const void *e, const void *s, const voi
     if (!ctx->bounce_buf) return fail(ctx, HRC_ESTATE, std::string(where) + ": call hrc_reserve_bounces first");
     if (K < 0 || K > ctx->bounce_cap)
         return fail(ctx, HRC_EINVAL, std::string(where) + ": bounces must be in [0, the count reserved by hrc_reserve_bounces]");
-    const Plan pl = f64 ? ctx->plan64 : own_config(ctx, ctx->plan);
+    const Plan pl = f64 ? ctx->plan64 : ctx->plan;
     const RayTable *rt = &ctx->rt;
     void *blur = ctx->blur ? ctx->blur_buf : nullptr;
     const double thr = ctx->blur_thr;
@@ -1473,7 +1488,7 @@ hrc_status bounces_backward(hrc_ctx *ctx, const void *gF, void *ge, void *gs, vo
     if (!gF || !ge || !gs || !ga) return fail(ctx, HRC_EINVAL, std::string(where) + ": NULL pointer");
     if (!aligned16(gF) || !aligned16(ge) || !aligned16(gs) || !aligned16(ga))
         return fail(ctx, HRC_EINVAL, std::string(where) + ": pointers must be 16-byte aligned");
-    const Plan pl = f64 ? ctx->plan64 : own_config(ctx, ctx->plan);
+    const Plan pl = f64 ? ctx->plan64 : ctx->plan;
     const RayTable *rt = &ctx->rt;
     void *blur = ctx->blur ? ctx->blur_buf : nullptr;
     const double thr = ctx->blur_thr;

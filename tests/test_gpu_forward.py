@@ -337,3 +337,35 @@ def test_trace_parts_in_fp64(W, H):
     from paper_2505_02041_gb300 import HRC
     F = HRC(W, H, 1, 0, "fp64").forward(to_dev(e), to_dev(s)).cpu().numpy()
     assert err_max(F, oracle.fluence(e, s)) <= 1e-10
+
+
+def test_launch_configuration_reads_back_what_runs():
+    """The configuration read from a context is the one its kernels run in:
+    writing it back, or copying it to another context, changes nothing (the
+    captured graph is replayed), on either side of 384^2 pixels, in every
+    precision and with per-channel extinction."""
+    require_gpu()
+    from paper_2505_02041_gb300 import HRC, _lib
+    small, large = dict(schedule=0, groups=1, threads=128, vmajor=0, mdown=0), dict(schedule=0, groups=4, threads=128,
+                                                                                     vmajor=1, mdown=0)
+    for W, H, prec, own in [(383, 384, "fp32", small), (384, 384, "fp32", large), (384, 384, "fp64", small),
+                            (400, 390, "bf16", large), (16384, 16, "fp32", dict(large, vmajor=0))]:
+        h = HRC(W, H, 1, 0, prec)
+        assert h.launch_config == own, (W, H, prec)
+        dt = torch.float64 if prec == "fp64" else torch.float32
+        e, s = (to_dev(x, dt) for x in scenes.random_scene(W, H, 1, 97))
+        out = torch.empty_like(e)
+        h.forward(e, s, out)
+        n = _lib.hrc_graph_captures(h.ctx)
+        h.set_launch_config(**h.launch_config)
+        h.forward(e, s, out)
+        assert _lib.hrc_graph_captures(h.ctx) == n and h.launch_config == own, (W, H, prec)
+    h = HRC(400, 390, 2)
+    h.set_precision("fp64")
+    h.set_channel_extinction(True)
+    assert h.launch_config == small
+    h.set_precision("fp32")
+    assert h.launch_config == large
+    h.set_launch_config(1, 2, 64, 0, 1)
+    h.set_precision("fp64")
+    assert h.launch_config == dict(schedule=1, groups=2, threads=64, vmajor=0, mdown=1)
