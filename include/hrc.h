@@ -328,8 +328,8 @@ hrc_status hrc_bounce_source(hrc_ctx *ctx, const float *emission, const float *s
 hrc_status hrc_sync(hrc_ctx *ctx);
 
 /* Test hook for the bounded device-side waits: with extra_bytes > 0
- * (0..4096) the trace and the mdown = 1 merge down arm their copy barriers
- * with that many bytes more than they copy, and the mdown = 2 persistent
+ * (0..4096) the trace, its adjoint and the mdown = 1 merge down arm their copy
+ * barriers with that many bytes more than they copy, and the mdown = 2 persistent
  * merge down publishes no finished item, so their waits run out after
  * `limit_ns` (<= 0 restores the default, 2 s) and hrc_sync reports
  * HRC_ETIMEOUT instead of a kernel hanging.  {0, 0} restores normal

@@ -1055,14 +1055,16 @@ template <class IN> __host__ __device__ inline IN *adj_part(const Plan &pl, int 
 // both go to planes that k_adj_combine sums.
 // With tme / tms (fp32 inputs) the tile region is fetched by TMA tensor
 // copies; a copy wait that gives up records its code in the plan's status
-// word and leaves the tile's gradients unwritten.
+// word and leaves the tile's image gradients unwritten (a plane's part, which
+// k_adj_combine adds, becomes zero).
 // fmask: the pair's frames to take (bits 0, 1); add: add to ge / gs (pair 1
-// launched after pair 0) instead of writing them.
+// launched after pair 0) instead of writing them; part: ge / gs are planes.
 template <int P, int C, class IN>
 __device__ __forceinline__ void body_adj_trace(const Plan &pl, const IN *__restrict__ e, const IN *__restrict__ s,
                                                IN *__restrict__ ge, IN *__restrict__ gs, int pair, int bx, int by,
                                                unsigned char *smem, const CUtensorMap *tme = nullptr,
-                                               const CUtensorMap *tms = nullptr, int fmask = 3, bool add = false) {
+                                               const CUtensorMap *tms = nullptr, int fmask = 3, bool add = false,
+                                               bool part = false) {
     using A = typename Prec<P>::A;
     PairTile<A, C> tt(smem);
     const AdjSlots<A, C> sl{reinterpret_cast<A *>(smem + PairTile<A, C>::bytes())};
@@ -1074,9 +1076,18 @@ __device__ __forceinline__ void body_adj_trace(const Plan &pl, const IN *__restr
     if constexpr (sizeof(A) == 4) {
         if (tme) {
             __shared__ __align__(8) uint64_t bar;
-            const int code = tt.stage_tma(pair, x0, y0, tme, tms, &bar, pl.bulk_limit_ns);
+            const int code = tt.stage_tma(pair, x0, y0, tme, tms, &bar, pl.bulk_limit_ns, (unsigned)pl.bulk_extra_tx);
             if (code != 0) {
                 if (threadIdx.x == 0) atomicMax(pl.status, code);
+                const int nx = pair == 0 ? PT_U : PT_V;
+                for (int k = threadIdx.x; part && k < PT_U * PT_V; k += blockDim.x) {
+                    const int x = x0 + k % nx, y = y0 + k / nx;
+                    if (x >= W || y >= H) continue;
+                    const long long pix = (long long)y * W + x;
+#pragma unroll
+                    for (int c = 0; c < C; ++c) ge[c * HW + pix] = IN(0);
+                    gs[pix] = IN(0);
+                }
                 return;
             }
         } else {

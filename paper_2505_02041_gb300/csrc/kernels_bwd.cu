@@ -116,7 +116,7 @@ __global__ void __launch_bounds__(ADJ_THREADS, 3) k_adj_trace_all(Plan pl, const
         gs = adj_part<IN>(pl, q, 1);
     }
     body_adj_trace<P, C, IN>(pl, e, s, ge, gs, pair, t % nx, t / nx, tb_smem, use_tma ? (pair ? &me1 : &me0) : nullptr,
-                             use_tma ? (pair ? &ms1 : &ms0) : nullptr, FB == 2 ? 3 : 1 << half);
+                             use_tma ? (pair ? &ms1 : &ms0) : nullptr, FB == 2 ? 3 : 1 << half, false, FB == 1 || pair);
 }
 
 // dL/de and dL/dsigma from the planes of k_adj_trace_all: (q0 + q1) + (q2 + q3).

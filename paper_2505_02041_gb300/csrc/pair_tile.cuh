@@ -133,7 +133,7 @@ template <class A, int C> struct PairTile {
     // into registers first, then the planes are written.  Returns 0, or
     // kWaitTimeout / kWaitLost when the copy wait gave up.
     __device__ __forceinline__ int stage_tma(int pair, int x0, int y0, const CUtensorMap *tme, const CUtensorMap *tms,
-                                             uint64_t *bar, long long limit_ns) {
+                                             uint64_t *bar, long long limit_ns, unsigned extra_tx) {
         static_assert(sizeof(A) == 4, "fp32 staging");
         constexpr int BOX = PT_RU * PT_RV;
         constexpr int PER = (BOX + 255) / 256;
@@ -145,7 +145,7 @@ template <class A, int C> struct PairTile {
         }
         __syncthreads();
         if (threadIdx.x == 0) {
-            mbar_arrive_expect(bar, (unsigned)((C + 1) * BOX * sizeof(float)));
+            mbar_arrive_expect(bar, (unsigned)((C + 1) * BOX * sizeof(float)) + extra_tx);
 #pragma unroll
             for (int c = 0; c < C; ++c) tma_load_3d(stg + c * BOX, tme, x0 - PT_HALO, y0 - PT_HALO, c, bar);
             tma_load_2d(stg + C * BOX, tms, x0 - PT_HALO, y0 - PT_HALO, bar);

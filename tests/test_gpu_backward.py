@@ -286,3 +286,33 @@ def test_adjoint_trace_at_its_lines(W, H, C, prec):
     ge, gs = _gpu_grads(e, s, gF, prec)
     tol = 1e-10 if prec == "fp64" else 1e-4
     assert err_max(ge, ge_r) <= tol and err_max(gs, gs_r) <= tol
+
+
+@pytest.mark.parametrize("W,H,C,fill", [(64, 48, 2, 0.0), (400, 404, 1, 7.0)])
+def test_adjoint_trace_wait_times_out_and_recovers(W, H, C, fill):
+    """The adjoint trace waits on its copy barrier with a time limit: armed (test
+    hook) with bytes that never arrive, every tile gives up, hrc_sync reports
+    HRC_ETIMEOUT and no partial sum reaches the gradients -- with a frame per
+    block they are the sum of empty parts, with a pair per block they stay as
+    they were -- and the context then computes correctly."""
+    require_gpu()
+    from paper_2505_02041_gb300 import HRC, _lib
+    e, s = scenes.random_scene(W, H, C, 53)
+    gF = scenes.rng(54).normal(size=e.shape).astype(np.float32)
+    h = HRC(W, H, C)
+    ed, sd, gd = to_dev(e), to_dev(s), to_dev(gF)
+    h.forward(ed, sd)
+    ge, gs = torch.full_like(ed, 7.0), torch.full_like(sd, 7.0)
+    _lib.hrc_debug_bulk_wait(h.ctx, 16, 1_000_000)
+    h.forward(ed, sd)
+    _lib.hrc_fluence_backward(h.ctx, gd, ge, gs)
+    with pytest.raises(_lib.HRCError) as ex:
+        h.sync()
+    assert ex.value.status == _lib.HRC_ETIMEOUT
+    assert bool((ge == fill).all()) and bool((gs == fill).all())
+    _lib.hrc_debug_bulk_wait(h.ctx, 0, 0)
+    h.forward(ed, sd)
+    ge, gs = (t.cpu().numpy() for t in h.backward(gd))
+    h.sync()
+    ge_r, gs_r = oracle.fluence_adjoint(e, s, gF)
+    assert err_max(ge, ge_r) <= 1e-4 and err_max(gs, gs_r) <= 1e-4
