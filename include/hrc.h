@@ -472,7 +472,8 @@ int hrc_last_launch_count(const hrc_ctx *ctx);
  * hrc_get_timing synchronises the stream and fills up to `cap` records of
  * the last compute call; it returns the number of records (or -1 on error).
  * `kind`: 0 trace T_0..T_2, 1 merge up, 2 merge down, 3 fluence sum,
- * 4 adjoint sum, 5 adjoint merge down, 6 adjoint merge up, 7 adjoint trace,
+ * 4 adjoint sum, 5 adjoint merge down, 6 adjoint merge up, 7 adjoint trace
+ * (level 0, then level 1: the sum of its partial planes, or its second half),
  * 8 batched persistent kernel, 9 other, 10 cross blur, 11 adjoint cross blur,
  * 12 bounce source update, 13 its adjoint.  `bytes` is the launch's
  * algorithmic traffic (each array it consumes read once, each array it

@@ -310,7 +310,8 @@ static cudaError_t bwd_impl(const Plan &pl, const RayTable &rt, const void *e, c
         if (all) {
             const int room = 152 * (P == P_FP64 ? 1 : (C == 4 ? 2 : 3));
             const bool one = pl.solo && 2 * (n0 + n1) <= room;   // a frame per block
-            double by = img * (pl.C + 1) * ab * (one ? 10.0 : 5.0);   // the inputs, the planes written and read, the sums
+            const double planes = one ? 4.0 : 2.0;
+            double by = img * (pl.C + 1) * ab * (1.0 + planes);   // the inputs, the planes written
             for (int q = 0; q < 4; ++q)
                 for (int n = 0; n <= 2; ++n) by += gTbytes(q, n);
             rec->begin(K_ADJ_TRACE, 0, by);
@@ -322,20 +323,22 @@ static cudaError_t bwd_impl(const Plan &pl, const RayTable &rt, const void *e, c
             IN *geo = (IN *)ge, *gso = (IN *)gs;
             const long long nb = ((long long)(pl.C + 1) * pl.W * pl.H + 255) / 256;
             const unsigned cb = (unsigned)(nb < 2432 ? nb : 2432);
-            if (one) {
+            if (one)
                 k_adj_trace_all<P, C, IN, 1><<<2 * (n0 + n1), ADJ_THREADS, smem, st>>>(pl, ei, si, geo, gso, n0, n1, nx0, nx1,
                                                                                     m[0], m[1], m[2], m[3], use_tma);
-                k_adj_combine<C, IN, 1><<<cb, 256, 0, st>>>(pl, geo, gso);
-            } else {
+            else
                 k_adj_trace_all<P, C, IN, 2><<<n0 + n1, ADJ_THREADS, smem, st>>>(pl, ei, si, geo, gso, n0, n1, nx0, nx1, m[0],
                                                                               m[1], m[2], m[3], use_tma);
-                k_adj_combine<C, IN, 2><<<cb, 256, 0, st>>>(pl, geo, gso);
-            }
+            rec->end();
+            rec->begin(K_ADJ_TRACE, 1, img * (pl.C + 1) * ab * (planes + 1.0));   // the planes read, the sums
+            if (one) k_adj_combine<C, IN, 1><<<cb, 256, 0, st>>>(pl, geo, gso);
+            else k_adj_combine<C, IN, 2><<<cb, 256, 0, st>>>(pl, geo, gso);
             rec->end();
             *launches += 2;
         }
         for (int pair = 0; pair < 2 && !all; ++pair) {
-            double by = img * (pl.C + 1) * ab * (pair == 0 ? 1.0 : 2.0);   // pair 1 adds to the gradients
+            // the inputs, the gradients written; pair 1 adds to them
+            double by = img * (pl.C + 1) * ab * (pair == 0 ? 2.0 : 3.0);
             for (int q = 2 * pair; q < 2 * pair + 2; ++q)
                 for (int n = 0; n <= 2; ++n) by += gTbytes(q, n);
             dim3 grid(pair_tiles_x(pair, pl.W), pair_tiles_y(pair, pl.H));

@@ -316,3 +316,22 @@ def test_adjoint_trace_wait_times_out_and_recovers(W, H, C, fill):
     h.sync()
     ge_r, gs_r = oracle.fluence_adjoint(e, s, gF)
     assert err_max(ge, ge_r) <= 1e-4 and err_max(gs, gs_r) <= 1e-4
+
+
+@pytest.mark.parametrize("W,H,C", [(64, 48, 2), (400, 404, 1), (4, 2, 1)])
+def test_timing_records_cover_every_launch(W, H, C):
+    """The timing records' launches add up to the pass's launch count, one
+    record a launch in the modes that time single launches, forward and
+    backward, in each form of the adjoint trace."""
+    require_gpu()
+    from paper_2505_02041_gb300 import HRC, _lib
+    e, s = (to_dev(x) for x in scenes.random_scene(W, H, C, 55))
+    h = HRC(W, H, C)
+    for mode in (1, 2, 3):
+        _lib.hrc_set_timing(h.ctx, mode)
+        for run in (lambda: h.forward(e, s), lambda: h.backward(torch.ones_like(e), e, s)):
+            run()
+            recs = _lib.hrc_get_timing(h.ctx)
+            assert sum(r[4] for r in recs) == h.launch_count(), mode
+            assert mode == 3 or all(r[4] == 1 for r in recs)
+    _lib.hrc_set_timing(h.ctx, 0)
