@@ -552,7 +552,7 @@ __device__ __forceinline__ void body_adj_T0(const Plan &pl, const RowSplitB &rs,
 // the level above (n = 2 .. N-1); adj_T covers the others.
 __host__ __device__ inline bool adj_T_fused(int n, int N) { return n >= 2 && n <= N - 1; }
 
-template <int P, int C, int E, bool ENV = false>
+template <int P, int C, int E>
 __device__ __forceinline__ void body_adj_T(const Plan &pl, const RowSplitB &rs, int n, long long bx, int by) {
     using A = typename Prec<P>::A;
     int local;
@@ -571,7 +571,7 @@ __device__ __forceinline__ void body_adj_T(const Plan &pl, const RowSplitB &rs, 
         k = local - x * K;
     }
     A gL[E][C], gT[E];
-    adj_T_part<P, C, E, ENV>(pl, q, n, x, k, v, gL, gT);
+    adj_T_part<P, C, E, false>(pl, q, n, x, k, v, gL, gT);
     GTLevel<P, C> gTn(pl, q, n);
 #pragma unroll
     for (int l = 0; l < E; ++l)

@@ -178,9 +178,9 @@ template <class A, int C> struct TraceTile {
 // Tile steps along the axes of frame Q, known at compile time so that every
 // piece's shared-memory address is the probe's plus a constant, and the rays
 // of a column are picked by its residue mod 4 instead of ray by ray: the
-// kernel is bound by instruction issue (69 % of the slots at 1024^2), and this
-// cut it from 56.2 to 52.5 us there (C = 3, fp32) and from 189.5 to 177 us at
-// 2048^2.
+// kernel issued in 69 % of the slots at 1024^2 (54 % now, at three blocks per SM
+// by shared memory, 2.25 waves), and this cut it from 56.2 to 52.5 us there (C =
+// 3, fp32) and from 189.5 to 177 us at 2048^2.
 template <int Q> struct TraceFrame {
     static constexpr int sgn = (Q == 0 || Q == 2) ? 1 : -1;   // image step along u
     static constexpr int su = sgn * (Q < 2 ? 1 : TR_PITCH), sv = Q < 2 ? TR_PITCH : 1;

@@ -46,7 +46,7 @@ struct Plan {
     int W, H, C, prec;
     int sched;                       // 0: each launch covers all four frames; 1: frame by frame
     int mgroups;                     // merge up: 1 = a pair of v per thread, 2 = two pairs, 4 = four consecutive v
-    int mthreads;                    // merge kernels: threads per block for paired-v bodies
+    int mthreads;                    // merge kernels: threads per block (quads of many registers: at most 256)
     int vmajor;                      // merge kernels: 1 = v-blocks of a row are adjacent in launch order
     int mdown;                       // merge down: 0 = per-thread loads, 1 = rows staged by bulk copies,
                                      // 2 = every level in one persistent launch
@@ -410,12 +410,6 @@ template <int P, int C> struct TLevel {
         for (int c = 0; c < C; ++c) r.L[c] = to_acc(reinterpret_cast<const SL *>(g)[(long long)c * Vs + v]);
         r.t = to_acc(reinterpret_cast<const ST *>(g + (long long)C * Vs * sizeof(SL))[v]);
         return r;
-    }
-    __device__ __forceinline__ void store(int x, int k, int v, const Iv<P, C> &r) const {
-        char *g = row(x, k);
-#pragma unroll
-        for (int c = 0; c < C; ++c) reinterpret_cast<SL *>(g)[(long long)c * Vs + v] = from_acc<SL>(r.L[c]);
-        reinterpret_cast<ST *>(g + (long long)C * Vs * sizeof(SL))[v] = from_acc<ST>(r.t);
     }
     // entries v and v+1 (v even)
     __device__ __forceinline__ void load2(int x, int k, int v, Iv<P, C> &a, Iv<P, C> &b) const {

@@ -247,8 +247,8 @@ __global__ void __launch_bounds__(256) k_multi(const Plan *__restrict__ plans, c
     else if constexpr (KIND == MK_ADJ_SUM) body_adj_sum<P, C, IN>(pl, (const IN *)io + eoff[m.scene], vb, row, smem);
     else if constexpr (KIND == MK_ADJ_R2) body_adj_R<P, C, 2>(pl, m.rs, n, row, vb);
     else if constexpr (KIND == MK_ADJ_R1) body_adj_R<P, C, 1>(pl, m.rs, n, row, vb);
-    else if constexpr (KIND == MK_ADJ_T2) body_adj_T<P, C, 2, false>(pl, m.rs, n, row, vb);
-    else if constexpr (KIND == MK_ADJ_T1) body_adj_T<P, C, 1, false>(pl, m.rs, n, row, vb);
+    else if constexpr (KIND == MK_ADJ_T2) body_adj_T<P, C, 2>(pl, m.rs, n, row, vb);
+    else if constexpr (KIND == MK_ADJ_T1) body_adj_T<P, C, 1>(pl, m.rs, n, row, vb);
     else body_adj_merge_up<P, C, false>(pl, m.rs, n, row, vb);
 }
 

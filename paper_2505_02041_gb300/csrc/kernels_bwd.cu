@@ -38,10 +38,11 @@ __global__ void __launch_bounds__(512) k_adj_T0(Plan pl, RowSplitB rs) {
     body_adj_T0<P, C, ENV>(pl, rs, row, vb);
 }
 
-// Levels n >= 1: four v per thread.  These kernels issue in about 65 % of the
-// slots, most of it addresses and range tests, so a thread that shares them
-// over four entries is faster than one of two -- provided that a shifted
-// range is tested once for all its rows (rows4, shifted4, interval4): with a
+// Levels n >= 1: four v per thread.  With a pair of v these kernels issued in
+// about 65 % of the slots, most of it addresses and range tests, so a thread that
+// shares them over four entries is faster (40-46 % of the slots, waiting for
+// loads instead) -- provided that a shifted range is tested once for all its
+// rows (rows4, shifted4, interval4): with a
 // test per channel the merge-up reverse took 513 us instead of 387 (1024^2,
 // C = 3, fp32).  Pairs -> quads, us, C = 3 / C = 1 at 1024^2 fp32: merge-down
 // reverse 272 -> 247 / 188 -> 144, merge-up reverse 374 -> 366 / 260 -> 196;
@@ -174,12 +175,6 @@ dim3 row_grid_b(const Plan &pl, long long rows, int per_block) {
     for (int q = 0; q < 4; ++q) Vmax = pl.q[q].V > Vmax ? pl.q[q].V : Vmax;
     const unsigned vb = (unsigned)((Vmax + per_block - 1) / per_block);
     return pl.vmajor ? dim3(vb, (unsigned)rows) : dim3((unsigned)rows, vb);
-}
-
-int vblocks_b(const Plan &pl, int bs) {
-    int Vmax = 0;
-    for (int q = 0; q < 4; ++q) Vmax = pl.q[q].V > Vmax ? pl.q[q].V : Vmax;
-    return (Vmax + bs - 1) / bs;
 }
 
 }  // namespace

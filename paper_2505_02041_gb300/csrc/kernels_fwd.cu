@@ -118,12 +118,6 @@ static dim3 row_grid(const Plan &pl, long long rows, int per_block) {
     return pl.vmajor ? dim3(vb, (unsigned)rows) : dim3((unsigned)rows, vb);
 }
 
-static int vblocks(const Plan &pl, int bs) {
-    int Vmax = 0;
-    for (int q = 0; q < 4; ++q) Vmax = pl.q[q].V > Vmax ? pl.q[q].V : Vmax;
-    return (Vmax + bs - 1) / bs;
-}
-
 // Algorithmic bytes of T_n / R_n of frame q: the live entries only (column 0
 // of every level and the dead entries of T_0 / T_1 are never touched).
 static double t_entry_bytes(const Plan &pl) {
@@ -193,7 +187,6 @@ bool encode_image_maps(const Plan &pl, const void *e, const void *s, int box_x, 
 template <int P, int C>
 static cudaError_t fwd_impl(const Plan &pl, const RayTable &rt, const void *e, const void *s, void *F,
                             cudaStream_t st0, int *launches, Recorder *rec, bool with_sum, const Branches *br) {
-    const int bs = 256;
     const bool env = plan_has_env(pl);   // kernels compiled for an environment map
     int Nmax = 0;
     for (int q = 0; q < 4; ++q) Nmax = pl.q[q].N > Nmax ? pl.q[q].N : Nmax;

@@ -196,29 +196,6 @@ template <class A, int C> struct PairTile {
     }
 };
 
-// Frame geometry of a tile column: quadrant q of pair p, tile origin (x0,
-// y0); column c (along u) and lane (along v).
-struct PairGeom {
-    int u, v;          // frame coordinates of the pixel
-    int base;          // region offset of the pixel
-    int su;            // region step for +1 along u (+-PT_PITCH); +1 along v is +1
-    bool valid;        // pixel inside the image
-};
-
-__device__ __forceinline__ PairGeom pair_geom(const Plan &pl, int q, int x0, int y0, int c, int lane) {
-    PairGeom g;
-    const bool xu = q < 2;
-    const int tu = xu ? x0 : y0, tv = xu ? y0 : x0;
-    const int ext_u = xu ? pl.W : pl.H, ext_v = xu ? pl.H : pl.W;
-    const bool fwd = (q == 0 || q == 2);
-    g.valid = tu + c < ext_u && tv + lane < ext_v;
-    g.u = fwd ? tu + c : ext_u - 1 - (tu + c);
-    g.v = tv + lane;
-    g.base = (PT_HALO + c) * PT_PITCH + PT_HALO + lane;
-    g.su = fwd ? PT_PITCH : -PT_PITCH;
-    return g;
-}
-
 // Tile grid of a quadrant pair.
 __host__ __device__ inline int pair_tiles_x(int pair, int W) { return pair == 0 ? (W + PT_U - 1) / PT_U : (W + PT_V - 1) / PT_V; }
 __host__ __device__ inline int pair_tiles_y(int pair, int H) { return pair == 0 ? (H + PT_V - 1) / PT_V : (H + PT_U - 1) / PT_U; }
